@@ -78,8 +78,9 @@ typedef enum {
                                   mfbc_autotune chose) */
 #define MFBC_PATH_GENERAL 1    /* force the general (any integer weight) kernels */
 #define MFBC_PATH_LEVEL   2    /* require the unit-weight level kernels (INVALID if weighted) */
-#define MFBC_PATH_DIST    3    /* distance-ordered kernels for small integer weights
-                                  (INVALID when the largest weight exceeds 4096); n_b is at
+#define MFBC_PATH_DIST    3    /* distance-ordered kernels for small integer weights, one block
+                                  per source or, for few sources of a large graph, the whole
+                                  device per distance step (INVALID when the largest weight exceeds 4096); n_b is at
                                   most 4096 and n * n_b stays below 2^32 */
 #define MFBC_PATH_SMALL   4    /* persistent kernel for small unit-weight graphs: every batch
                                   of the call in one launch (INVALID if weighted or when
@@ -105,9 +106,11 @@ typedef struct {
   mfbc_kernel_stat k[MFBC_MAX_KSTATS];
   uint64_t batches;
   uint64_t fwd_iters;          /* MFBF products over all batches (distance kernels: distance
-                                  steps, including those that settle no pair) */
+                                  steps, including those that settle no pair; one block per
+                                  source: the steps of the longest source) */
   uint64_t bwd_iters;          /* MFBr products over all batches (distance kernels: steps that
-                                  settled pairs, distance 0 excepted) */
+                                  settled pairs, distance 0 excepted; one block per source:
+                                  as fwd_iters, MFBr running inside the same kernel) */
   int32_t n_b;                 /* batch width used */
   int32_t path;                /* MFBC_PATH_GENERAL, MFBC_PATH_LEVEL or MFBC_PATH_DIST */
   uint64_t stat[4];            /* with MFBC_OPT_COUNT_BYTES, level kernels: (neighbour, word)

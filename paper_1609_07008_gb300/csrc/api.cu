@@ -196,6 +196,9 @@ extern "C" mfbc_status mfbc_graph_info(const mfbc_graph* G, int32_t* n, int64_t*
 struct Plan {
   int path = MFBC_PATH_GENERAL;
   int nb = 32;
+  bool by_source = false;          // the call runs on the source kernel (source.cu):
+  SourcePlan src, wide;            //   its blocks and state, and its redo form
+  int redo_cap = 0;                //   sources a launch may hand to the redo form
   int groups = 0;                  // persistent small-graph kernel: block groups
   int64_t table_batches = 1;       //   and the batches its table holds
   int Lcap = 0;
@@ -228,11 +231,28 @@ static void level_caps(const DevGraph& g, int nb, int* Lcap, int64_t* list_cap) 
   *list_cap = n * std::min<int64_t>(*Lcap, 24) + 64;
 }
 
+// The source kernel's blocks and state: its form for the graph and, when that
+// keeps 16-bit distances, room for a launch's list of redone sources and for
+// the wide form (with as many blocks as fit) in the same memory.  most: at most
+// this many blocks (0: as planned).
+static void source_sizes(const DevGraph& g, int cols, int nb, int most, Plan* p) {
+  source_plan(g, cols, false, p->src);
+  source_plan(g, cols, true, p->wide);
+  if (most > 0) p->src.slots = std::min(p->src.slots, most);
+  p->redo_cap = p->src.dm != p->wide.dm ? nb : 0;
+  const size_t have = p->src.slot_bytes * (size_t)p->src.slots;
+  p->wide.slots = (int)std::max<size_t>(1, std::min<size_t>((size_t)p->wide.slots, have / p->wide.slot_bytes));
+  p->state_bytes = std::max(source_bytes(p->src, p->redo_cap), source_bytes(p->wide, p->redo_cap));
+}
+
 static size_t plan_bytes(const DevGraph& g, int path, int nb, int32_t nsrc, int mode, bool host_io,
-                         Plan* p) {
+                         Plan* p, bool by_source = false, int most = 0) {
   p->path = path;
   p->nb = nb;
-  if (path == MFBC_PATH_LEVEL) {
+  p->by_source = by_source;
+  if (by_source) {
+    source_sizes(g, std::min(nb, std::max(nsrc, 1)), nb, most, p);
+  } else if (path == MFBC_PATH_LEVEL) {
     level_caps(g, nb, &p->Lcap, &p->list_cap);
     // room for the general kernels at n_b = 32 too: the fallback used when
     // a batch is deeper than the level capacity runs in the same scratch
@@ -272,13 +292,45 @@ static bool small_graph(const DevGraph& g) { return g.n <= (1 << 13) && g.nnz <=
 // graphs on which mfbc_autotune also times the persistent kernel
 static bool small_tunable(const DevGraph& g) { return g.n <= (1 << 15) && g.nnz <= (1 << 19); }
 
+static bool has_hubs(const DevGraph& g) {
+  return std::max(g.max_deg, g.max_in_deg) > std::max<int64_t>(64, 4 * (g.n ? g.nnz / g.n : 0));
+}
+
 static int default_path(const DevGraph& g) {
   if (g.unit) return small_graph(g) ? MFBC_PATH_SMALL : MFBC_PATH_LEVEL;
-  const int64_t avg = g.n ? g.nnz / g.n : 0;
-  const int64_t deg_cap = std::max<int64_t>(64, 4 * avg);
-  if (g.wmax <= 128 && std::max(g.max_deg, g.max_in_deg) <= deg_cap && (uint64_t)g.n * 128u <= 0xffffffffull)
+  if (g.wmax <= 128 && !has_hubs(g) && (uint64_t)g.n * 128u <= 0xffffffffull)
     return MFBC_PATH_DIST;
   return MFBC_PATH_GENERAL;
+}
+
+// The source kernel (source.cu) or the kernels of the family, for the distance
+// kernels and for calls of the general kernels that leave the choice open
+// (MFBC_PATH_AUTO, untuned, no accumulator named).
+//
+// A source on one block takes about 4 us per distance value that occurs plus
+// its arcs' share, however few sources run.  The distance kernels spread a step
+// over the whole GPU, which wins where few sources meet wide steps: uniform
+// n = 300 000, k = 16, weights <= 20, 1 / 8 / 32 / 48 sources 10.3 / 10.9 / 12.3
+// / 13.2 ms here against 2.4 / 4.5 / 9.3 / 14.4 there; n = 10^6, k = 8: 25 / 29 /
+// 33 / 35 against 3.5 / 10 / 24 / 38; n = 100 000, k = 32, weights <= 100, 1 / 8
+// sources 6.0 / 6.1 against 5.2 / 6.6.  On lattices (degrees <= 8) the steps are
+// narrow and the blocks win from one source on: weighted 256^2 grid, 1 / 64 /
+// 256 sources 7.1 / 10.8 / 13 ms against 24 / 49 / 58.
+static bool dist_by_source(const DevGraph& g, int32_t nsrc) {
+  if (std::max(g.max_deg, g.max_in_deg) <= 8) return true;
+  return !((g.n >= (1 << 18) && nsrc <= 40) || (g.n >= (1 << 16) && nsrc <= 4));
+}
+// The general kernels' time goes with their 15-25 Bellman-Ford products (0.1-0.3
+// ms each and up) whatever the weights are, the source kernel's with the
+// distance values, of which larger weights make more.  R-MAT 14, weights <= 255,
+// 2 / 128 / 1024 sources: 1.7 / 1.7 / 7.7 ms against 6.6 / 9.0 / 39; uniform
+// n = 100 000, k = 8, weights <= 255, 1 / 8 / 48 sources 4.5 / 4.5 / 4.9 against
+// 3.2 / 4.8 / 9.1; weights <= 1000, 2 / 128 / 1024 sources: 14.5 / 18.8 / 52
+// against 3.6 / 18.1 / 155; R-MAT 14, weights <= 4000, 128 / 1024 sources: 14 /
+// 57 against 12 / 44.
+static bool general_by_source(const DevGraph& g, int32_t nsrc) {
+  if (g.unit || (uint64_t)g.n * 128u > 0xffffffffull || g.wmax > 1024) return false;
+  return nsrc >= (g.wmax > 256 ? 128 : has_hubs(g) ? 1 : 8);
 }
 
 static int tuned_slot(int path) {
@@ -308,6 +360,28 @@ static mfbc_status make_plan(const mfbc_graph* G, int32_t nsrc, int mode, const 
     maxnb = (int)std::min<int64_t>(maxnb, cap);
     if (maxnb < 32) return fail(MFBC_ERR_INVALID, "MFBC_PATH_DIST needs n < 2^27");
   }
+  // may the source kernel take the call, and does the rule choose it?
+  const bool open_general = path == MFBC_PATH_GENERAL && (!opt || (opt->path == MFBC_PATH_AUTO && !opt->accumulator)) &&
+                            !G->tuned_path && !G->tuned_arcs && !G->tuned_accum && !G->force_arcs;
+  const bool can_source = path == MFBC_PATH_DIST || (open_general && general_by_source(g, INT32_MAX));
+  const bool by_source =
+      can_source && (path == MFBC_PATH_DIST ? dist_by_source(g, nsrc) : general_by_source(g, nsrc));
+  // A source plan is cut down to fewer blocks where its scratch does not fit; the
+  // family's kernels take over when not even one block's does.
+  auto fit_source = [&](int nb, size_t room) {
+    if (p->total <= room) return;
+    const size_t rest = p->total - p->src.slot_bytes * (size_t)p->src.slots;
+    const int most = room > rest ? (int)((room - rest) / p->src.slot_bytes) : 0;
+    plan_bytes(g, path, nb, nsrc, mode, host_io, p, true, std::max(most, 1));
+    if (p->total > room) plan_bytes(g, path, nb, nsrc, mode, host_io, p);
+  };
+  // The family's kernels do not fit a caller's workspace: the source kernel may
+  // (a workspace sized for more sources, where the rule chose it).
+  auto try_source = [&](int nb, size_t room) {
+    if (!can_source || p->by_source || p->total <= room) return;
+    plan_bytes(g, path, nb, nsrc, mode, host_io, p, true);
+    fit_source(nb, room);
+  };
   // the level kernels move 128 columns (four 32-column words) at a time
   const int gran = path == MFBC_PATH_LEVEL ? 128 : 32;
   int req = opt ? opt->n_b : 0;
@@ -320,7 +394,18 @@ static mfbc_status make_plan(const mfbc_graph* G, int32_t nsrc, int mode, const 
   if (req > 0) {
     int nb = (req + gran - 1) / gran * gran;
     if (nb > maxnb) return fail(MFBC_ERR_INVALID, "n_b too large for this path (max " + std::to_string(maxnb) + ")");
-    plan_bytes(g, path, nb, nsrc, mode, host_io, p);
+    plan_bytes(g, path, nb, nsrc, mode, host_io, p, by_source);
+    // the narrowest width, which callers short of memory come down to, asks for
+    // no more state than 24 bytes per vertex and column
+    if (by_source && nb == gran) fit_source(nb, p->extra_bytes + 24ull * (size_t)g.n * nb + (size_t)(64 << 10));
+    if (opt->workspace) {
+      if (by_source) fit_source(nb, opt->workspace_bytes);
+      else try_source(nb, opt->workspace_bytes);
+    } else if (by_source && p->total > G->ws_bytes) {      // the cached scratch would grow: within the device's room
+      size_t fr = 0, tot = 0;
+      if (cudaMemGetInfo(&fr, &tot) == cudaSuccess) fit_source(nb, (size_t)(0.80 * (double)(fr + G->ws_bytes)));
+      else cudaGetLastError();
+    }
     return MFBC_OK;
   }
   // auto: widest batch (<= number of sources, <= the tuned width) whose
@@ -334,20 +419,24 @@ static mfbc_status make_plan(const mfbc_graph* G, int32_t nsrc, int mode, const 
     budget = (size_t)(0.80 * (double)(fr + G->ws_bytes));
   }
   // the persistent small-graph kernel runs batches side by side: 128 columns
-  // per batch leave it several batches to spread over its block groups.  On
-  // dense graphs (average degree >= 64) the distance kernels check one
-  // 4-byte distance per in-arc and pair, each in its own 32-byte sector, so
-  // a batch whose distances stay in the L2 wins: dense weighted ER n = 2^16,
-  // k = 1024, 4096 sources, n_b 256 / 512 / 1024 / 4096: 64.9 / 66.0 /
-  // 62.3 / 51.5 GTEPS
-  const bool dense_dist = path == MFBC_PATH_DIST && g.nnz >= 64 * (int64_t)std::max(g.n, 1);
-  const int widest = tuned > 0 ? tuned : (path == MFBC_PATH_SMALL ? 128 : dense_dist ? std::min(maxnb, 512) : maxnb);
+  // per batch leave it several batches to spread over its block groups
+  const int widest = tuned > 0 ? tuned : (path == MFBC_PATH_SMALL ? 128 : maxnb);
   int nb = std::min(widest, std::max(gran, (nsrc + gran - 1) / gran * gran));
+  if (by_source) {
+    int b = nb;
+    for (;; b -= gran) {
+      plan_bytes(g, path, b, nsrc, mode, host_io, p, true);
+      if (p->total <= budget || b == gran) break;
+    }
+    fit_source(b, budget);
+    if (p->by_source) return MFBC_OK;
+  }
   while (true) {
     plan_bytes(g, path, nb, nsrc, mode, host_io, p);
     if (p->total <= budget || nb == gran) break;
     nb -= gran;
   }
+  if (opt && opt->workspace) try_source(nb, budget);
   return MFBC_OK;
 }
 
@@ -669,6 +758,69 @@ mfbc_status small_path(mfbc_graph* G, Run& R, RunCtx& rc, SmallState& ss, const 
   return MFBC_OK;
 }
 
+// Every source of the call on the source kernel: it takes them from a queue,
+// and those it lists (a distance past 16 bits) run again in the wide form.  n_b
+// bounds the sources of a launch where rows, lists or staged outputs have room
+// for that many.  d_row: room for n_b lambda rows (mode 2).
+mfbc_status source_path(Run& R, RunCtx& rc, const int32_t* d_src, int32_t nsrc, int mode, double* d_lambda,
+                      int32_t* dist_out, double* sigma_out, bool out_on_host, const int32_t* lrows, int32_t* d_row,
+                      int32_t* stage_d, double* stage_s, uint32_t* warn, int64_t* fi, int64_t* bi) {
+  const DevGraph& g = *rc.g;
+  const Plan& P = R.plan;
+  SourceState ss, sw;
+  Carver c1(R.ws, R.ws_bytes), c2(R.ws, R.ws_bytes);
+  source_carve(c1, P.src, P.redo_cap, ss);
+  source_carve(c2, P.wide, P.redo_cap, sw);  // the same counters and list, other block states
+  std::vector<int32_t> rows;
+  if (mode == 2)
+    for (int32_t r = 0; r < R.nreq; r++)
+      rows.insert(rows.end(), (size_t)(R.req_off[r + 1] - R.req_off[r]), lrows ? lrows[r] : r);
+  MFBC_CUDA_TRY(cudaMemsetAsync(ss.ctl, 0, sizeof(SrcCtl), R.st), rc.err);
+  const bool chunked = P.redo_cap || mode == 2 || (mode == 1 && out_on_host);
+  const int32_t step = chunked ? P.nb : std::max(nsrc, 1);
+  SrcCtl* h = (SrcCtl*)rc.h_ctr;
+  for (int32_t b0 = 0; b0 < nsrc; b0 += step) {
+    const int32_t na = std::min(step, nsrc - b0);
+    if (mode == 2)
+      MFBC_CUDA_TRY(cudaMemcpyAsync(d_row, rows.data() + b0, sizeof(int32_t) * (size_t)na, cudaMemcpyHostToDevice,
+                                    R.st), rc.err);
+    int32_t* dd = mode != 1 ? nullptr : out_on_host ? stage_d : dist_out + (size_t)b0 * g.n;
+    double* ds = mode != 1 || !sigma_out ? nullptr : out_on_host ? stage_s : sigma_out + (size_t)b0 * g.n;
+    double* lam = mode == 1 ? nullptr : d_lambda;
+    mfbc_status s = source_run(rc, P.src, ss, d_src + b0, mode == 2 ? d_row : nullptr, nullptr, na, lam, dd, ds,
+                               K_DP_FWD);
+    if (s) return s;
+    if (P.redo_cap || b0 + step >= nsrc) {
+      MFBC_CUDA_TRY(cudaMemcpyAsync(h, ss.ctl, sizeof(SrcCtl), cudaMemcpyDeviceToHost, R.st), rc.err);
+      MFBC_CUDA_TRY(cudaStreamSynchronize(R.st), rc.err);
+      rc.prof->drain();
+      if (h->nredo) {
+        const int32_t nr = (int32_t)h->nredo;
+        MFBC_CUDA_TRY(cudaMemsetAsync(&ss.ctl->nredo, 0, sizeof(uint32_t), R.st), rc.err);
+        s = source_run(rc, P.wide, sw, d_src + b0, mode == 2 ? d_row : nullptr, ss.redo, nr, lam, dd, ds, K_DP_FWD);
+        if (s) return s;
+        MFBC_CUDA_TRY(cudaMemcpyAsync(h, ss.ctl, sizeof(SrcCtl), cudaMemcpyDeviceToHost, R.st), rc.err);
+        MFBC_CUDA_TRY(cudaStreamSynchronize(R.st), rc.err);
+        rc.prof->drain();
+      }
+    }
+    if (mode == 1 && out_on_host) {
+      MFBC_CUDA_TRY(cudaMemcpyAsync(dist_out + (size_t)b0 * g.n, stage_d, sizeof(int32_t) * (size_t)na * g.n,
+                                    cudaMemcpyDeviceToHost, R.st), rc.err);
+      if (sigma_out)
+        MFBC_CUDA_TRY(cudaMemcpyAsync(sigma_out + (size_t)b0 * g.n, stage_s, sizeof(double) * (size_t)na * g.n,
+                                      cudaMemcpyDeviceToHost, R.st), rc.err);
+      MFBC_CUDA_TRY(cudaStreamSynchronize(R.st), rc.err);
+    }
+  }
+  if (nsrc) {
+    if (h->flags & FLAG_SIGMA_INEXACT) *warn |= MFBC_WARN_SIGMA_INEXACT;
+    *fi += h->steps;                           // of the longest source
+    if (mode != 1) *bi += h->steps;
+  }
+  return MFBC_OK;
+}
+
 // mode 0: lambda (d_lambda device, n doubles, overwritten); mode 1: sssp rows;
 // mode 2: one lambda row per request (d_lambda device, nreq * n doubles).
 mfbc_status run(mfbc_graph* G, const int32_t* d_src, int32_t nsrc, int mode, double* d_lambda,
@@ -685,9 +837,11 @@ mfbc_status run(mfbc_graph* G, const int32_t* d_src, int32_t nsrc, int mode, dou
   GeneralState gs;
   LevelState ls;
   DistState ds;
+  SourceState srcs;
   Counters* ctr;
   SmallState ss;
-  if (P.path == MFBC_PATH_LEVEL) { level_carve(c, g, nb, P.Lcap, P.list_cap, ls); ctr = ls.ctr; }
+  if (P.by_source) { source_carve(c, P.src, P.redo_cap, srcs); ctr = srcs.ctr; }
+  else if (P.path == MFBC_PATH_LEVEL) { level_carve(c, g, nb, P.Lcap, P.list_cap, ls); ctr = ls.ctr; }
   else if (P.path == MFBC_PATH_DIST) { dist_carve(c, g.n, nb, g.wmax + 1, ds); ctr = ds.ctr; }
   else if (P.path == MFBC_PATH_SMALL) { small_carve(c, g.n, nb, P.groups, ss); ctr = ss.ctr; }
   else { general_carve(c, g.n, nb, gs); ctr = gs.ctr; }
@@ -746,7 +900,14 @@ mfbc_status run(mfbc_graph* G, const int32_t* d_src, int32_t nsrc, int mode, dou
     if (so) return fail(so, R.err.empty() ? std::string(mfbc_status_string(so)) : R.err);
     if (applied) d_src = d_sorted;
   }
-  for (int64_t bx = 0; bx < (P.path == MFBC_PATH_SMALL ? 0 : nbatches); bx++) {
+  if (P.by_source && g.n) {
+    mfbc_status s = source_path(R, rc, d_src, nsrc, mode, d_lambda, dist_out, sigma_out, out_on_host, lrows, d_colidx,
+                              stage_d, stage_s, &warn, &fi, &bi);
+    if (s) return fail(s, R.err.empty() ? std::string(mfbc_status_string(s)) : R.err);
+    batches = nbatches;
+  }
+  const bool batched = !P.by_source && P.path != MFBC_PATH_SMALL;
+  for (int64_t bx = 0; bx < (batched ? nbatches : 0); bx++) {
     const int32_t b0 = multi ? 0 : (int32_t)(bx * nb);
     int na;
     const int32_t* bsrc;
@@ -851,7 +1012,7 @@ mfbc_status run(mfbc_graph* G, const int32_t* d_src, int32_t nsrc, int mode, dou
                                       cudaMemcpyDeviceToHost, R.st), &R.err);
     }
   }
-  if (P.path != MFBC_PATH_SMALL) {            // the small path read its flags already
+  if (batched) {                              // the other paths have read their flags
     MFBC_CUDA_TRY(cudaMemcpyAsync(G->h_ctr, &ctr->flags, sizeof(uint32_t), cudaMemcpyDeviceToHost, R.st), &R.err);
     MFBC_CUDA_TRY(cudaStreamSynchronize(R.st), &R.err);
     if (G->h_ctr[0] & FLAG_SIGMA_INEXACT) warn |= MFBC_WARN_SIGMA_INEXACT;

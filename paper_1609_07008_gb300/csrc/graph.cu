@@ -155,6 +155,37 @@ static mfbc_status upload_hot_targets(DevGraph* g, const std::vector<int64_t>& r
   return MFBC_OK;
 }
 
+// out[k] = col[k] | w[k] << bits
+__global__ void k_pack_arcs(const int32_t* __restrict__ col, const int32_t* __restrict__ w, int64_t nnz, int bits,
+                            uint32_t* __restrict__ out) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < nnz; k += stride)
+    out[k] = (uint32_t)col[k] | ((uint32_t)w[k] << bits);
+}
+
+// Column and weight of a weighted graph's arc in one word, for the source
+// kernel (half the bytes and one load an arc).  They always fit: distances are
+// int32, so n * w_max < 2^31, and with n > 2^(cb-1), w_max >= 2^(wb-1) the bits
+// cb + wb are at most 32.
+static mfbc_status pack_arcs(DevGraph* g, cudaStream_t st, std::string* err) {
+  int cb = 1, wb = 1;
+  while ((1ll << cb) < g->n) cb++;
+  while ((1ll << wb) <= g->wmax) wb++;
+  if (!g->w) return MFBC_OK;
+  if (cb + wb > 32) { *err = "column and weight of an arc do not fit in 32 bits"; return MFBC_ERR_OVERFLOW; }
+  g->pk_bits = cb;
+  const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>((g->nnz + 255) / 256, 152 * 16));
+  TRY(dev_alloc(g, &g->pk, (size_t)g->nnz, err));
+  k_pack_arcs<<<blocks, 256, 0, st>>>(g->col, g->w, g->nnz, cb, g->pk);
+  g->pk_t = g->pk;
+  if (g->directed) {
+    TRY(dev_alloc(g, &g->pk_t, (size_t)g->nnz, err));
+    k_pack_arcs<<<blocks, 256, 0, st>>>(g->col_t, g->w_t, g->nnz, cb, g->pk_t);
+  }
+  MFBC_CUDA_TRY(cudaStreamSynchronize(st), err);
+  return MFBC_OK;
+}
+
 mfbc_status graph_build(int32_t n, int64_t nnz, const int64_t* h_rowptr, const int32_t* h_col,
                         const int32_t* h_w, uint32_t flags, cudaStream_t st, DevGraph* g,
                         std::string* err) {
@@ -262,7 +293,7 @@ mfbc_status graph_build(int32_t n, int64_t nnz, const int64_t* h_rowptr, const i
     g->col_t = g->col;
     g->w_t = g->w;
   }
-  return MFBC_OK;
+  return pack_arcs(g, st, err);
 }
 
 void graph_free(DevGraph* g) {

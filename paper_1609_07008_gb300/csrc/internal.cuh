@@ -51,6 +51,9 @@ struct DevGraph {
   int64_t* rowptr_t = nullptr;     // CSR of A^T (in-arcs); aliases CSR when undirected
   int32_t* col_t = nullptr;
   int32_t* w_t = nullptr;
+  uint32_t* pk = nullptr;          // A's arcs as column | weight << pk_bits (nullptr when unit)
+  uint32_t* pk_t = nullptr;        //   and those of A^T (aliases pk when undirected)
+  int pk_bits = 0;
   ItemList items_in;               // over A^T rows (MFBF pull gathers in-arcs)
   ItemList items_out;              // over A rows   (MFBr pull gathers out-arcs)
   std::vector<void*> owned;        // device allocations to free
@@ -210,6 +213,35 @@ struct DistState {
 size_t dist_bytes(int32_t n, int nb, int B);
 void dist_carve(Carver& c, int32_t n, int nb, int B, DistState& s);
 
+// Source path: one block per source, for weighted graphs in order of distance
+// value and for small unit-weight graphs by levels.  See source.cu.
+struct SourcePlan {
+  int dm = 0, am = 0;    // where tau lives, how arcs are stored (DM_*, AM_* of source.cu)
+  int threads = 128, slots = 1;   // block size, blocks (one state each)
+  int B = 0;             // buckets (w_max + 1) of cap entries, scap of them in shared memory
+  uint32_t scap = 0, cap = 0;
+  size_t smem = 0, slot_bytes = 0;
+  uint32_t dcap = 0;     // DAG arcs kept per source
+  size_t o_dist = 0, o_sv = 0, o_z = 0, o_order = 0, o_ring = 0, o_dag = 0;   // offsets within a slot
+};
+struct SrcCtl {          // read back once per call
+  uint32_t head;         // source queue
+  uint32_t nredo;        // sources listed for the wide form
+  uint32_t steps;        // most steps of a source
+  uint32_t flags;        // FLAG_* bits
+};
+struct SourceState {
+  char* slots;           // [slots] block states of slot_bytes
+  SrcCtl* ctl;
+  int32_t* redo;         // sources for the wide form
+  Counters* ctr;
+};
+// Blocks and state for at most `cols` sources in flight; wide: the form without
+// 16-bit distances, which sources that outgrow them are redone in.
+void source_plan(const DevGraph& g, int cols, bool wide, SourcePlan& p);
+size_t source_bytes(const SourcePlan& p, int32_t nredo);
+void source_carve(Carver& c, const SourcePlan& p, int32_t nredo, SourceState& s);
+
 // Persistent path for small unit-weight graphs: whole batches inside one
 // cooperative launch, block groups taking batches from a device queue.  See
 // small.cu.
@@ -278,6 +310,14 @@ mfbc_status level_output(RunCtx& rc, LevelState& s, int levels, int nactive, int
 mfbc_status dist_batch(RunCtx& rc, DistState& s, const int32_t* d_src_batch, int nactive, double* lambda,
                        int64_t* fwd_iters, int64_t* bwd_iters);
 mfbc_status dist_output(RunCtx& rc, DistState& s, int nactive, int32_t* dist_out, double* sigma_out);
+
+// The sources d_src[0 .. nsrc) -- or, with d_list, d_src[d_list[0 .. nsrc)] --
+// on the source kernel, launched once and not waited for.  d_row: lambda row of
+// each source or null (row 0).  lambda null: MFBF only, source i writing row i
+// of dist_out / sigma_out.
+mfbc_status source_run(RunCtx& rc, const SourcePlan& p, SourceState& s, const int32_t* d_src, const int32_t* d_row,
+                       const int32_t* d_list, int32_t nsrc, double* lambda, int32_t* dist_out, double* sigma_out,
+                       KId id);
 
 // All batches of a call on the persistent small-graph kernel.  d_src_all:
 // [nbatch][nb] columns' sources (-1 padding); d_wreq: [nbatch][W] lambda row
