@@ -71,8 +71,8 @@ typedef enum {
 #define MFBC_WARN_SIGMA_INEXACT 1u  /* some sigma_bar >= 2^53: FP64 counts may be rounded */
 
 /* mfbc_options.path */
-#define MFBC_PATH_AUTO    0    /* unit weights: the persistent small-graph kernel when n <= 2^13
-                                  and nnz <= 2^18, else the level kernels; distance kernels for weights
+#define MFBC_PATH_AUTO    0    /* unit weights: MFBC_PATH_SMALL when n <= 2^13 and nnz <= 2^18,
+                                  else the level kernels; distance kernels for weights
                                   <= 128 when no in- or out-degree exceeds max(64, 4x the
                                   average degree); general kernels otherwise (or the family
                                   mfbc_autotune chose) */
@@ -82,9 +82,8 @@ typedef enum {
                                   per source or, for few sources of a large graph, the whole
                                   device per distance step (INVALID when the largest weight exceeds 4096); n_b is at
                                   most 4096 and n * n_b stays below 2^32 */
-#define MFBC_PATH_SMALL   4    /* persistent kernel for small unit-weight graphs: every batch
-                                  of the call in one launch (INVALID if weighted or when
-                                  n * n_b * 9 bytes per group does not fit; see below) */
+#define MFBC_PATH_SMALL   4    /* small unit-weight graphs: every source of the call in one
+                                  launch, one block per source (INVALID if weighted) */
 
 typedef struct mfbc_graph mfbc_graph;   /* opaque, device resident */
 

@@ -210,9 +210,9 @@ struct Plan {
 
 static inline size_t al256(size_t b) { return (b + 255) & ~size_t(255); }
 
-static size_t extras(const DevGraph& g, int32_t nsrc, int mode, int nb, bool host_io, int path) {
+static size_t extras(const DevGraph& g, int32_t nsrc, int mode, int nb, bool host_io, int path, bool by_source) {
   size_t b = 0;
-  if (path == MFBC_PATH_SMALL) {             // the call's batch table: sources, lambda rows, packed columns
+  if (path == MFBC_PATH_SMALL && !by_source) {   // the call's batch table: sources, lambda rows, packed columns
     const size_t nbatch = std::max<size_t>(1, ((size_t)nsrc + nb - 1) / nb);
     b += 2 * al256(sizeof(int32_t) * nbatch * nb) + al256(sizeof(int32_t) * nbatch * (nb / 32));
   }
@@ -220,7 +220,8 @@ static size_t extras(const DevGraph& g, int32_t nsrc, int mode, int nb, bool hos
   if (host_io) b += al256(sizeof(int32_t) * (size_t)std::max(nsrc, 1));        // device sources
   if (mode == 0) b += al256(sizeof(int32_t) * (size_t)std::max(nsrc, 1));      // reordered sources
   if (mode == 1 && host_io) b += al256((sizeof(int32_t) + sizeof(double)) * (size_t)nb * std::max(g.n, 1));
-  if (mode == 2) b += 2 * al256(sizeof(int32_t) * (size_t)nb);                 // packed batch columns
+  if (mode == 2 && by_source) b += al256(sizeof(int32_t) * (size_t)std::max(nsrc, 1));   // lambda row of each source
+  else if (mode == 2) b += 2 * al256(sizeof(int32_t) * (size_t)nb);            // packed batch columns
   return b;
 }
 
@@ -232,14 +233,14 @@ static void level_caps(const DevGraph& g, int nb, int* Lcap, int64_t* list_cap) 
 }
 
 // The source kernel's blocks and state: its form for the graph and, when that
-// keeps 16-bit distances, room for a launch's list of redone sources and for
+// keeps narrow distances or counts, room for a list of redone sources and for
 // the wide form (with as many blocks as fit) in the same memory.  most: at most
 // this many blocks (0: as planned).
-static void source_sizes(const DevGraph& g, int cols, int nb, int most, Plan* p) {
-  source_plan(g, cols, false, p->src);
-  source_plan(g, cols, true, p->wide);
+static void source_sizes(const DevGraph& g, bool unit, int cols, int32_t nsrc, int most, Plan* p) {
+  source_plan(g, cols, unit, false, p->src);
+  source_plan(g, cols, unit, true, p->wide);
   if (most > 0) p->src.slots = std::min(p->src.slots, most);
-  p->redo_cap = p->src.dm != p->wide.dm ? nb : 0;
+  p->redo_cap = p->src.unit || p->src.dm != p->wide.dm ? nsrc : 0;
   const size_t have = p->src.slot_bytes * (size_t)p->src.slots;
   p->wide.slots = (int)std::max<size_t>(1, std::min<size_t>((size_t)p->wide.slots, have / p->wide.slot_bytes));
   p->state_bytes = std::max(source_bytes(p->src, p->redo_cap), source_bytes(p->wide, p->redo_cap));
@@ -251,7 +252,10 @@ static size_t plan_bytes(const DevGraph& g, int path, int nb, int32_t nsrc, int 
   p->nb = nb;
   p->by_source = by_source;
   if (by_source) {
-    source_sizes(g, std::min(nb, std::max(nsrc, 1)), nb, most, p);
+    // (on the unit-weight path n_b does not bound the sources in flight: a
+    // block's state is small, and the blocks share nothing)
+    const bool unit = path == MFBC_PATH_SMALL || path == MFBC_PATH_LEVEL;
+    source_sizes(g, unit, unit ? std::max(nsrc, 1) : std::min(nb, std::max(nsrc, 1)), nsrc, most, p);
   } else if (path == MFBC_PATH_LEVEL) {
     level_caps(g, nb, &p->Lcap, &p->list_cap);
     // room for the general kernels at n_b = 32 too: the fallback used when
@@ -269,7 +273,7 @@ static size_t plan_bytes(const DevGraph& g, int path, int nb, int32_t nsrc, int 
   } else {
     p->state_bytes = general_bytes(g.n, nb);
   }
-  p->extra_bytes = extras(g, nsrc, mode, nb, host_io, path);
+  p->extra_bytes = extras(g, nsrc, mode, nb, host_io, path, by_source);
   p->total = p->state_bytes + p->extra_bytes;
   return p->total;
 }
@@ -333,6 +337,19 @@ static bool general_by_source(const DevGraph& g, int32_t nsrc) {
   return nsrc >= (g.wmax > 256 ? 128 : has_hubs(g) ? 1 : 8);
 }
 
+// The level kernels share a frontier's bit rows and arcs among the columns of a
+// batch but pay 1.2 ms of launches for a batch however small; one block per
+// source pays every arc for every source.  Milliseconds level / source kernel
+// at 1, 64, 152, 304, 456 sources: R-MAT 14 (4.3 * 10^5 arcs) 1.4 / 0.5, 1.8 /
+// 0.7, 2.0 / 0.7, 2.2 / 1.2, 2.4 / 2.0; uniform n = 20 000, k = 60 1.3 / 1.1,
+// 1.8 / 1.2, 2.2 / 1.2, 2.6 / 2.3, 3.1 / 4.4; uniform n = 60 000, k = 8 2.0 /
+// 1.0, 2.6 / 1.0, 3.0 / 1.3, 3.7 / 3.0, 4.3 / 6.1; directed R-MAT 16 (9.6 * 10^5)
+// 1.7 / 1.3, 2.2 / 1.7, 2.6 / 1.8, 3.3 / 3.4; R-MAT 16 (1.8 * 10^6) 1.8 / 2.3,
+// 2.8 / 2.5; uniform n = 16 000, k = 10, 500 / 2000 sources 2.2 / 1.3, 5.8 / 4.7.
+static bool level_by_source(const DevGraph& g, int32_t nsrc) {
+  return g.nnz <= 1250000 && (nsrc <= 152 || (int64_t)nsrc * g.nnz <= 130000000);
+}
+
 static int tuned_slot(int path) {
   return path == MFBC_PATH_LEVEL ? 0 : path == MFBC_PATH_GENERAL ? 1 : path == MFBC_PATH_DIST ? 2 : 3;
 }
@@ -363,9 +380,14 @@ static mfbc_status make_plan(const mfbc_graph* G, int32_t nsrc, int mode, const 
   // may the source kernel take the call, and does the rule choose it?
   const bool open_general = path == MFBC_PATH_GENERAL && (!opt || (opt->path == MFBC_PATH_AUTO && !opt->accumulator)) &&
                             !G->tuned_path && !G->tuned_arcs && !G->tuned_accum && !G->force_arcs;
-  const bool can_source = path == MFBC_PATH_DIST || (open_general && general_by_source(g, INT32_MAX));
-  const bool by_source =
-      can_source && (path == MFBC_PATH_DIST ? dist_by_source(g, nsrc) : general_by_source(g, nsrc));
+  const bool small = path == MFBC_PATH_SMALL && !(opt && (opt->flags & MFBC_OPT_TEST_STALL));
+  const bool open_level = path == MFBC_PATH_LEVEL && !G->tuned_path && !G->tuned_nb[0] &&
+                          (!opt || (opt->path == MFBC_PATH_AUTO && !(opt->flags & MFBC_OPT_TEST_SMALL_ROUNDS)));
+  const bool can_source = g.nnz < (1ll << 31) && (path == MFBC_PATH_DIST || small || (open_general && general_by_source(g, INT32_MAX)) ||
+                                                  (open_level && level_by_source(g, 1)));
+  const bool by_source = can_source && (small || (path == MFBC_PATH_DIST    ? dist_by_source(g, nsrc)
+                                                  : path == MFBC_PATH_LEVEL ? level_by_source(g, nsrc)
+                                                                            : general_by_source(g, nsrc)));
   // A source plan is cut down to fewer blocks where its scratch does not fit; the
   // family's kernels take over when not even one block's does.
   auto fit_source = [&](int nb, size_t room) {
@@ -420,7 +442,7 @@ static mfbc_status make_plan(const mfbc_graph* G, int32_t nsrc, int mode, const 
   }
   // the persistent small-graph kernel runs batches side by side: 128 columns
   // per batch leave it several batches to spread over its block groups
-  const int widest = tuned > 0 ? tuned : (path == MFBC_PATH_SMALL ? 128 : maxnb);
+  const int widest = tuned > 0 ? tuned : (path == MFBC_PATH_SMALL && !by_source ? 128 : maxnb);
   int nb = std::min(widest, std::max(gran, (nsrc + gran - 1) / gran * gran));
   if (by_source) {
     int b = nb;
@@ -759,52 +781,50 @@ mfbc_status small_path(mfbc_graph* G, Run& R, RunCtx& rc, SmallState& ss, const 
 }
 
 // Every source of the call on the source kernel: it takes them from a queue,
-// and those it lists (a distance past 16 bits) run again in the wide form.  n_b
-// bounds the sources of a launch where rows, lists or staged outputs have room
-// for that many.  d_row: room for n_b lambda rows (mode 2).
+// and those it lists (a distance or path count past its narrow form) run again
+// in the wide form.  Host outputs of mode 1 are staged n_b rows at a time.
+// d_row: room for the lambda row of each source (mode 2).
 mfbc_status source_path(Run& R, RunCtx& rc, const int32_t* d_src, int32_t nsrc, int mode, double* d_lambda,
-                      int32_t* dist_out, double* sigma_out, bool out_on_host, const int32_t* lrows, int32_t* d_row,
-                      int32_t* stage_d, double* stage_s, uint32_t* warn, int64_t* fi, int64_t* bi) {
+                        int32_t* dist_out, double* sigma_out, bool out_on_host, const int32_t* lrows, int32_t* d_row,
+                        int32_t* stage_d, double* stage_s, uint32_t* warn, int64_t* fi, int64_t* bi) {
   const DevGraph& g = *rc.g;
   const Plan& P = R.plan;
+  const KId id = P.src.unit ? K_SMALL : K_DP_FWD;
   SourceState ss, sw;
   Carver c1(R.ws, R.ws_bytes), c2(R.ws, R.ws_bytes);
   source_carve(c1, P.src, P.redo_cap, ss);
   source_carve(c2, P.wide, P.redo_cap, sw);  // the same counters and list, other block states
   std::vector<int32_t> rows;
-  if (mode == 2)
+  if (mode == 2 && nsrc) {
+    rows.reserve((size_t)nsrc);
     for (int32_t r = 0; r < R.nreq; r++)
       rows.insert(rows.end(), (size_t)(R.req_off[r + 1] - R.req_off[r]), lrows ? lrows[r] : r);
+    MFBC_CUDA_TRY(cudaMemcpyAsync(d_row, rows.data(), sizeof(int32_t) * (size_t)nsrc, cudaMemcpyHostToDevice, R.st),
+                  rc.err);
+  }
   MFBC_CUDA_TRY(cudaMemsetAsync(ss.ctl, 0, sizeof(SrcCtl), R.st), rc.err);
-  const bool chunked = P.redo_cap || mode == 2 || (mode == 1 && out_on_host);
-  const int32_t step = chunked ? P.nb : std::max(nsrc, 1);
+  const bool staged = mode == 1 && out_on_host;
+  const int32_t step = staged ? P.nb : std::max(nsrc, 1);
   SrcCtl* h = (SrcCtl*)rc.h_ctr;
   for (int32_t b0 = 0; b0 < nsrc; b0 += step) {
     const int32_t na = std::min(step, nsrc - b0);
-    if (mode == 2)
-      MFBC_CUDA_TRY(cudaMemcpyAsync(d_row, rows.data() + b0, sizeof(int32_t) * (size_t)na, cudaMemcpyHostToDevice,
-                                    R.st), rc.err);
-    int32_t* dd = mode != 1 ? nullptr : out_on_host ? stage_d : dist_out + (size_t)b0 * g.n;
-    double* ds = mode != 1 || !sigma_out ? nullptr : out_on_host ? stage_s : sigma_out + (size_t)b0 * g.n;
+    int32_t* dd = mode != 1 ? nullptr : staged ? stage_d : dist_out;
+    double* ds = mode != 1 || !sigma_out ? nullptr : staged ? stage_s : sigma_out;
     double* lam = mode == 1 ? nullptr : d_lambda;
-    mfbc_status s = source_run(rc, P.src, ss, d_src + b0, mode == 2 ? d_row : nullptr, nullptr, na, lam, dd, ds,
-                               K_DP_FWD);
+    mfbc_status s = source_run(rc, P.src, ss, d_src + b0, mode == 2 ? d_row : nullptr, nullptr, na, lam, dd, ds, id);
     if (s) return s;
-    if (P.redo_cap || b0 + step >= nsrc) {
+    for (bool again = true; again;) {
       MFBC_CUDA_TRY(cudaMemcpyAsync(h, ss.ctl, sizeof(SrcCtl), cudaMemcpyDeviceToHost, R.st), rc.err);
       MFBC_CUDA_TRY(cudaStreamSynchronize(R.st), rc.err);
       rc.prof->drain();
-      if (h->nredo) {
-        const int32_t nr = (int32_t)h->nredo;
-        MFBC_CUDA_TRY(cudaMemsetAsync(&ss.ctl->nredo, 0, sizeof(uint32_t), R.st), rc.err);
-        s = source_run(rc, P.wide, sw, d_src + b0, mode == 2 ? d_row : nullptr, ss.redo, nr, lam, dd, ds, K_DP_FWD);
-        if (s) return s;
-        MFBC_CUDA_TRY(cudaMemcpyAsync(h, ss.ctl, sizeof(SrcCtl), cudaMemcpyDeviceToHost, R.st), rc.err);
-        MFBC_CUDA_TRY(cudaStreamSynchronize(R.st), rc.err);
-        rc.prof->drain();
-      }
+      again = h->nredo != 0;                 // the wide form lists none
+      if (!again) break;
+      MFBC_CUDA_TRY(cudaMemsetAsync(&ss.ctl->nredo, 0, sizeof(uint32_t), R.st), rc.err);
+      s = source_run(rc, P.wide, sw, d_src + b0, mode == 2 ? d_row : nullptr, ss.redo, (int32_t)h->nredo, lam, dd, ds,
+                     id);
+      if (s) return s;
     }
-    if (mode == 1 && out_on_host) {
+    if (staged) {
       MFBC_CUDA_TRY(cudaMemcpyAsync(dist_out + (size_t)b0 * g.n, stage_d, sizeof(int32_t) * (size_t)na * g.n,
                                     cudaMemcpyDeviceToHost, R.st), rc.err);
       if (sigma_out)
@@ -814,8 +834,9 @@ mfbc_status source_path(Run& R, RunCtx& rc, const int32_t* d_src, int32_t nsrc, 
     }
   }
   if (nsrc) {
+    if (h->flags & FLAG_BAD_SOURCE) { *rc.err = "source id out of range"; return MFBC_ERR_INVALID; }
     if (h->flags & FLAG_SIGMA_INEXACT) *warn |= MFBC_WARN_SIGMA_INEXACT;
-    *fi += h->steps;                           // of the longest source
+    *fi += h->steps;                         // of the longest source
     if (mode != 1) *bi += h->steps;
   }
   return MFBC_OK;
@@ -848,7 +869,8 @@ mfbc_status run(mfbc_graph* G, const int32_t* d_src, int32_t nsrc, int mode, dou
   int32_t* stage_d = nullptr;
   double* stage_s = nullptr;
   char* small_tab = extra;
-  if (P.path == MFBC_PATH_SMALL) {          // batch table first (see extras)
+  const bool small = P.path == MFBC_PATH_SMALL && !P.by_source;
+  if (small) {          // batch table first (see extras)
     const size_t nbatch = (size_t)P.table_batches;
     extra += 2 * al256(sizeof(int32_t) * nbatch * nb) + al256(sizeof(int32_t) * nbatch * (nb / 32));
   }
@@ -873,20 +895,20 @@ mfbc_status run(mfbc_graph* G, const int32_t* d_src, int32_t nsrc, int mode, dou
   Packing pk;
   int32_t* d_colidx = nullptr;
   int32_t* d_batch = nullptr;
-  if (multi) {
+  if (multi) d_colidx = (int32_t*)extra;     // (by source: the lambda rows)
+  if (multi && !P.by_source) {
     pk = pack_requests(R.req_off, R.nreq, nb, lrows);
-    d_colidx = (int32_t*)extra;
     d_batch = (int32_t*)(extra + al256(sizeof(int32_t) * (size_t)nb));
   }
-  const int64_t nbatches = multi ? pk.batches : ((int64_t)nsrc + nb - 1) / nb;
+  const int64_t nbatches = multi && !P.by_source ? pk.batches : ((int64_t)nsrc + nb - 1) / nb;
   uint32_t warn = 0;
-  if (P.path == MFBC_PATH_SMALL) {
+  if (small) {
     mfbc_status s = small_path(G, R, rc, ss, d_src, nsrc, mode, d_lambda, dist_out, sigma_out, out_on_host, pk,
                                nbatches, small_tab, stage_d, stage_s, &warn, &fi, &bi);
     if (s) return fail(s, R.err.empty() ? std::string(mfbc_status_string(s)) : R.err);
     batches = nbatches;
   }
-  if (P.path == MFBC_PATH_LEVEL && g.n) {
+  if (P.path == MFBC_PATH_LEVEL && !P.by_source && g.n) {
     // masks start clean; each batch returns them to zero
     MFBC_CUDA_TRY(cudaMemsetAsync(ls.V, 0, sizeof(uint32_t) * (size_t)g.n * ls.W, R.st), &R.err);
     MFBC_CUDA_TRY(cudaMemsetAsync(ls.F, 0, sizeof(uint32_t) * (size_t)ls.Lcap * g.n * ls.W, R.st), &R.err);
@@ -894,7 +916,7 @@ mfbc_status run(mfbc_graph* G, const int32_t* d_src, int32_t nsrc, int mode, dou
     if (g.items_out.nhub)
       MFBC_CUDA_TRY(cudaMemsetAsync(ls.zacc, 0, sizeof(double) * (size_t)g.items_out.nhub * nb, R.st), &R.err);
   }
-  if (mode == 0 && P.path == MFBC_PATH_LEVEL && nsrc > nb && !(R.opt && (R.opt->flags & MFBC_OPT_KEEP_ORDER))) {
+  if (mode == 0 && P.path == MFBC_PATH_LEVEL && !P.by_source && nsrc > nb && !(R.opt && (R.opt->flags & MFBC_OPT_KEEP_ORDER))) {
     bool applied = false;
     mfbc_status so = order_sources(rc, ls, d_src, nsrc, d_sorted, &applied);
     if (so) return fail(so, R.err.empty() ? std::string(mfbc_status_string(so)) : R.err);
@@ -906,7 +928,7 @@ mfbc_status run(mfbc_graph* G, const int32_t* d_src, int32_t nsrc, int mode, dou
     if (s) return fail(s, R.err.empty() ? std::string(mfbc_status_string(s)) : R.err);
     batches = nbatches;
   }
-  const bool batched = !P.by_source && P.path != MFBC_PATH_SMALL;
+  const bool batched = !P.by_source && !small;
   for (int64_t bx = 0; bx < (batched ? nbatches : 0); bx++) {
     const int32_t b0 = multi ? 0 : (int32_t)(bx * nb);
     int na;
@@ -1091,7 +1113,7 @@ mfbc_status entry(const mfbc_graph* Gc, const int32_t* sources, int32_t nsrc, in
   // only the level kernels' gathers gain from the 32-byte fetch hint; setting
   // and restoring it costs two driver calls that small calls would feel
   std::optional<L2FetchHint> l2hint;
-  if (R.plan.path == MFBC_PATH_LEVEL) l2hint.emplace();
+  if (R.plan.path == MFBC_PATH_LEVEL && !R.plan.by_source) l2hint.emplace();
   R.prof.on = opt && opt->profile;
   R.prof.count_bytes = R.prof.on && (opt->flags & MFBC_OPT_COUNT_BYTES);
   R.prof.stream = R.st;

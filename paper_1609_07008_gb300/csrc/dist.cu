@@ -24,6 +24,11 @@
 // A step reads each item's 32 distances with one warp and works the pairs at
 // its distance one per lane; the items that settle pairs are appended to one
 // list with per-step offsets, which the backward pass replays in reverse.
+//
+// These kernels spread one step of all sources over the whole device.  The
+// source kernel (source.cu: a block per source, no launch per step) takes
+// every call but few sources of a large graph; the rule and both sides'
+// figures are in api.cu.
 #include <algorithm>
 
 #include "internal.cuh"

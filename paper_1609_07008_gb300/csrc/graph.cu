@@ -182,6 +182,7 @@ static mfbc_status pack_arcs(DevGraph* g, cudaStream_t st, std::string* err) {
     TRY(dev_alloc(g, &g->pk_t, (size_t)g->nnz, err));
     k_pack_arcs<<<blocks, 256, 0, st>>>(g->col_t, g->w_t, g->nnz, cb, g->pk_t);
   }
+  // (calls on the graph may come on any stream: everything is there at return)
   MFBC_CUDA_TRY(cudaStreamSynchronize(st), err);
   return MFBC_OK;
 }

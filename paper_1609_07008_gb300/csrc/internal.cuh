@@ -216,13 +216,14 @@ void dist_carve(Carver& c, int32_t n, int nb, int B, DistState& s);
 // Source path: one block per source, for weighted graphs in order of distance
 // value and for small unit-weight graphs by levels.  See source.cu.
 struct SourcePlan {
+  bool unit = false;     // by levels, 64-bit counts
   int dm = 0, am = 0;    // where tau lives, how arcs are stored (DM_*, AM_* of source.cu)
   int threads = 128, slots = 1;   // block size, blocks (one state each)
   int B = 0;             // buckets (w_max + 1) of cap entries, scap of them in shared memory
   uint32_t scap = 0, cap = 0;
   size_t smem = 0, slot_bytes = 0;
   uint32_t dcap = 0;     // DAG arcs kept per source
-  size_t o_dist = 0, o_sv = 0, o_z = 0, o_order = 0, o_ring = 0, o_dag = 0;   // offsets within a slot
+  size_t o_dist = 0, o_cell = 0, o_order = 0, o_ring = 0, o_dag = 0;   // offsets within a slot
 };
 struct SrcCtl {          // read back once per call
   uint32_t head;         // source queue
@@ -236,9 +237,10 @@ struct SourceState {
   int32_t* redo;         // sources for the wide form
   Counters* ctr;
 };
-// Blocks and state for at most `cols` sources in flight; wide: the form without
-// 16-bit distances, which sources that outgrow them are redone in.
-void source_plan(const DevGraph& g, int cols, bool wide, SourcePlan& p);
+// Blocks and state for at most `cols` sources in flight; unit: by levels with
+// 64-bit counts; wide: the form without narrow distances or counts, which
+// sources that outgrow them are redone in.
+void source_plan(const DevGraph& g, int cols, bool unit, bool wide, SourcePlan& p);
 size_t source_bytes(const SourcePlan& p, int32_t nredo);
 void source_carve(Carver& c, const SourcePlan& p, int32_t nredo, SourceState& s);
 

@@ -28,16 +28,29 @@
 // flight rather than by one step's vertices.
 //
 // What bounds it: the latency of a step (a chain of five or six dependent loads
-// and one atomic, about 3 us) where steps are narrow, the walk over the arcs
-// where they are wide.  MFBr does not walk the arcs again: MFBF records every
-// DAG arc it finds (on average one to two per vertex), and MFBr replays them
-// backwards, so that only zeta of a vertex is loaded in a step's chain.
-// Measured against one launch per step for all sources (distance kernels) or
-// Bellman-Ford products (general kernels), one call: weighted 256^2 grid, 512
-// sources 67.0 -> 12.4 ms; uniform n = 2^15, k = 512, weights <= 100, 300
-// sources 47.6 -> 9.4 ms (5 * 10^9 arcs, each read once: 2.1 TB/s of packed
-// arcs out of the L2); directed R-MAT 16, weights <= 255, 2048 sources 209 ->
-// 50.9 ms.
+// and one atomic, 2.5 us) where steps are narrow; the instructions of the walk
+// over the arcs (44 a warp and 32 arcs) where they are wide.  MFBr does not
+// walk the arcs again: MFBF records every DAG arc it finds, and MFBr replays
+// them backwards, so that only zeta of a vertex is loaded in a step's chain.
+//
+// Measured, one call, against one launch per step for all sources (distance
+// kernels), Bellman-Ford products (general kernels) and block groups that meet
+// at a barrier after each level of 128 sources (small-graph kernel): weighted
+// 256^2 grid, 512 sources 67.0 -> 11.9 ms; uniform n = 2^15, k = 512, weights
+// <= 100, 300 sources 47.6 -> 8.7 ms (5 * 10^9 arcs, each read once: 2.3 TB/s
+// of packed arcs out of the L2); directed R-MAT 16, weights <= 255, 2048
+// sources 209 -> 48 ms; uniform n = 1024, k = 8, all sources 0.58 -> 0.21 ms;
+// R-MAT 13, 500 sources 5.3 -> 1.0 ms; unit-weight 60^2 grid, 500 sources 111 ->
+// 1.2 ms (its batches were too deep or their counts too large for the
+// small-graph kernel and went to the general kernels).
+//
+// Tried and not kept: a chunk of a step's rows laid end to end and cut into
+// equal spans for the block's warps (no hub rows, perfect balance): R-MAT 14
+// unit weights 3.3 -> 5.2 ms, directed weighted R-MAT 16 47 -> 53 ms, weighted
+// 256^2 grid 11.9 -> 11.5 ms; the rows' scan, two barriers and the per-arc row
+// search cost more than the balance gives.  One block of 128-512 threads and
+// several sources an SM with tau in global memory on power-law graphs (139 ms
+// against 48): the sources' tau rows fall out of the L2.
 #include <algorithm>
 #include <type_traits>
 
@@ -54,9 +67,9 @@ constexpr int SRC_SMEM_MAX = 226 * 1024;
 constexpr int SRC_SMS = 152;
 __host__ __device__ constexpr size_t src_al16(size_t b) { return (b + 15) & ~size_t(15); }
 
-// Where tau lives (DM): 32 bits in global memory, 32 bits in shared memory, or
-// 16 bits in shared memory (a source with a distance past 65534 is redone).
-constexpr int DM_GLOBAL = 0, DM_SMEM32 = 1, DM_SMEM16 = 2;
+// Where tau lives (DM): 32 bits in global memory; 32, 16 or, for unit weights, 8
+// bits in shared memory (a source with a distance past 65534 or 254 is redone).
+constexpr int DM_GLOBAL = 0, DM_SMEM32 = 1, DM_SMEM16 = 2, DM_SMEM8 = 3;
 // How arcs are stored (AM): column only (unit weights), or column and weight
 // packed in 32 bits.
 constexpr int AM_UNIT = 0, AM_PACKED = 1;
@@ -92,9 +105,8 @@ struct SrcArgs {
   double* sigma_out;
   char* slots;                         // [gridDim.x] block states, slot_bytes apart
   size_t slot_bytes;
-  size_t o_dist, o_sv, o_z, o_order, o_ring, o_dag;  // offsets within a slot
-  uint32_t dcap;                       // DAG arcs a slot holds (weighted)
-  int so;                              // the queue and the step offsets are in shared memory
+  size_t o_dist, o_cell, o_order, o_ring, o_dag;  // offsets within a slot
+  uint32_t dcap;                       // DAG arcs a slot holds
   int B;                               // buckets (weighted): w_max + 1
   uint32_t scap, cap;                  // entries of a bucket in shared memory, and in all
   SrcCtl* ctl;
@@ -102,11 +114,9 @@ struct SrcArgs {
   unsigned long long* bytes;           // algorithmic bytes (counting runs), or null
 };
 
-// A vertex's reduction in one step, kept in 8 bytes of shared memory.  F64:
-// FP64 sums (weighted graphs; path counts are integers below 2^53, exact in
-// any order).  DF: unit weights, exact 64-bit counts and compensated
-// double-float values (dfloat.cuh).  seg() adds up runs of equal, non-decreasing
-// keys over the warp; the last lane of a run then holds its sum.
+// A vertex's reduction in one step, kept in 8 bytes of shared memory: FP64 sums
+// (values, and path counts of weighted graphs: integers below 2^53, exact in any
+// order) or exact 64-bit counts (unit weights).
 struct SumF64 {
   double s = 0.0;
   __device__ __forceinline__ static SumF64 of_count(uint64_t x) { return {__longlong_as_double((long long)x)}; }
@@ -124,16 +134,6 @@ struct SumU64 {
   __device__ __forceinline__ void add(const SumU64& o) { i += o.i; }
   __device__ __forceinline__ SumU64 up(int o) const { return {__shfl_up_sync(0xffffffffu, i, o)}; }
 };
-struct SumDF {
-  float s = 0.f, c = 0.f;
-  __device__ __forceinline__ static SumDF of_value(uint64_t x) { const dfl v = df_unpack(x); return {v.hi, v.lo}; }
-  __device__ __forceinline__ uint64_t bits() const { return df_pack({s, c}); }
-  __device__ __forceinline__ void add(const SumDF& o) { acc_add(s, c, o.s, o.c); }
-  __device__ __forceinline__ SumDF up(int o) const {
-    return {__shfl_up_sync(0xffffffffu, s, o), __shfl_up_sync(0xffffffffu, c, o)};
-  }
-};
-
 template <int ILP>
 struct SrcWarp {
   uint64_t acc[32];                    // sums of the batch's 32 vertices
@@ -141,28 +141,62 @@ struct SrcWarp {
   uint8_t t[32 + 32 * ILP];            //   and the vertex's place in the batch
 };
 
+// sigma_bar (an integer or an FP64 count; in the pulled form of MFBr later the
+// value zeta + 1/sigma_bar) and zeta of a vertex, side by side: a vertex costs
+// one 32-byte sector of the L2 rather than one for each.
+struct SrcCell {
+  uint64_t sv;
+  double z;
+};
+
 // The state of one source in one block.
 template <int DM>
 struct SrcState {
-  using D = typename std::conditional<DM == DM_SMEM16, uint16_t, int32_t>::type;
+  using D = typename std::conditional<DM == DM_SMEM8, uint8_t,
+                                      typename std::conditional<DM == DM_SMEM16, uint16_t, int32_t>::type>::type;
+  static constexpr int32_t NONE = DM == DM_SMEM8 ? 0xff : DM == DM_SMEM16 ? 0xffff : INF;   // unreached
   SrcShared& sh;
   uint32_t* cnt;                       // bucket counts (weighted)
   int32_t* sring;                      // [B][scap] first entries of each bucket
   D* dist;                             // tau
-  uint64_t* sv;                        // sigma_bar, then zeta + 1/sigma_bar
+  SrcCell* cell;                       // sigma_bar and zeta
   int32_t* order;                      // vertices in settling order
-  uint32_t* off;                       // first entry of each step; weighted: (order, dag) pairs
+  uint2* off;                          // first entries of each step in order and dag
   int32_t* ring;                       // [B][cap - scap] further bucket entries (weighted)
-  double* z;                           // zeta (weighted)
-  int2* dag;                           // DAG arcs as (vertex, predecessor), in step order (weighted)
+  // DAG arcs as (vertex, predecessor), in step order; two 16-bit ids in a word
+  // where every id fits (dag16)
+  uint32_t* dag;
+  bool dag16;
+  __device__ __forceinline__ void put_arc(uint32_t at, int32_t v, int32_t u) {
+    if (dag16) dag[at] = (uint32_t)v | ((uint32_t)u << 16);
+    else reinterpret_cast<int2*>(dag)[at] = make_int2(v, u);
+  }
+  __device__ __forceinline__ int2 arc(uint32_t at) const {
+    if (!dag16) return reinterpret_cast<const int2*>(dag)[at];
+    const uint32_t x = dag[at];
+    return make_int2((int32_t)(x & 0xffffu), (int32_t)(x >> 16));
+  }
   __device__ __forceinline__ int32_t tau(int32_t v) const {
-    const D x = dist[v];
-    return DM == DM_SMEM16 && x == (D)0xffff ? INF : (int32_t)x;
+    const int32_t x = (int32_t)dist[v];
+    return x == NONE ? INF : x;
+  }
+  // unit weights: gives v the level l unless it has one; true for the caller
+  // that did.  Every caller of a step offers the same level, so clearing the
+  // bits that l lacks from an unreached entry (all ones) sets it once.
+  __device__ __forceinline__ bool claim(int32_t v, int32_t l) {
+    if constexpr (DM == DM_SMEM8 || DM == DM_SMEM16) {
+      constexpr int per = 4 / (int)sizeof(D);
+      uint32_t* word = reinterpret_cast<uint32_t*>(dist) + v / per;
+      const int shift = (v % per) * 8 * (int)sizeof(D);
+      const uint32_t old = atomicAnd(word, ~((uint32_t)(NONE ^ l) << shift));
+      return ((old >> shift) & (uint32_t)NONE) == (uint32_t)NONE;
+    } else {
+      return atomicMin(&dist[v], l) > l;
+    }
   }
   // lowers tau(v) to cand; true for the caller that did
   __device__ __forceinline__ bool lower(int32_t v, int32_t cand) {
     if constexpr (DM == DM_SMEM16) {
-      if (cand >= 0xffff) { sh.redo = 1u; return false; }
       unsigned short* p = reinterpret_cast<unsigned short*>(&dist[v]);
       unsigned short old = *reinterpret_cast<volatile unsigned short*>(p);
       while ((int32_t)old > cand) {
@@ -171,6 +205,8 @@ struct SrcState {
         old = seen;
       }
       return false;
+    } else if constexpr (DM == DM_SMEM8) {
+      return false;                    // unit weights only: see claim
     } else {
       return atomicMin(&dist[v], cand) > cand;
     }
@@ -179,34 +215,36 @@ struct SrcState {
 
 // Sums the list's first 32 entries (qn of them when fewer) into the batch's
 // accumulators.  Entries are grouped by vertex.
-template <class Sum, bool COUNT, bool RECORD, int ILP, class S>
+template <class Sum, bool COUNT, int ILP, class S>
 __device__ __forceinline__ void src_flush(const SrcArgs& a, SrcWarp<ILP>& wb, S& st, int q0, int qn, int32_t mv) {
   const unsigned lane = lane_id();
   const bool has = (int)lane < qn;
   const int t = has ? (int)wb.t[q0 + lane] : 64;
   Sum x;
   const int32_t y = has ? wb.y[q0 + lane] : 0;
-  if (RECORD) {                        // the DAG arc, for MFBr
+  if (COUNT) {                         // MFBF: the DAG arc, for MFBr
     uint32_t at = 0;
     if (lane == 0) at = atomicAdd(&st.sh.dtail, (uint32_t)qn);
     at = __shfl_sync(0xffffffffu, at, 0) + lane;
     const int32_t v = __shfl_sync(0xffffffffu, mv, t & 31);
-    if (has && at < a.dcap) st.dag[at] = make_int2(v, y);
+    if (has && at < a.dcap) st.put_arc(at, v, y);
   }
   if (has) {
-    const uint64_t b = st.sv[y];
+    const uint64_t b = st.cell[y].sv;
     if constexpr (COUNT) x = Sum::of_count(b);
     else x = Sum::of_value(b);
   }
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    if (o >= qn) break;                // (uniform) no run is longer than the list
+  // sum of each run of one vertex, on the run's last lane, in as many steps as
+  // the longest run needs
+  const int tp = __shfl_up_sync(0xffffffffu, t, 1);
+  const uint32_t heads = __ballot_sync(0xffffffffu, lane == 0 || tp != t) | 1u;
+  const int back = (int)lane - (31 - __clz(heads & (0xffffffffu >> (31u - lane))));   // lanes to the run's first
+  const int longest = (int)__reduce_max_sync(0xffffffffu, has ? (unsigned)back : 0u);
+  for (int o = 1; o <= longest; o <<= 1) {
     const Sum x2 = x.up(o);
-    const int t2 = __shfl_up_sync(0xffffffffu, t, o);
-    if ((int)lane >= o && t2 == t) x.add(x2);
+    if (back >= o) x.add(x2);
   }
-  const int tn = __shfl_down_sync(0xffffffffu, t, 1);
-  if (has && (lane == 31 || tn != t)) {
+  if (has && ((int)lane == qn - 1 || ((heads >> (lane + 1)) & 1u))) {
     Sum sum;
     if constexpr (COUNT) sum = Sum::of_count(wb.acc[t]);
     else sum = Sum::of_value(wb.acc[t]);
@@ -216,37 +254,41 @@ __device__ __forceinline__ void src_flush(const SrcArgs& a, SrcWarp<ILP>& wb, S&
   __syncwarp();
 }
 
-template <int AM>
-__device__ __forceinline__ void src_arc(const SrcArgs& a, const uint32_t* __restrict__ arc, int64_t k, bool in,
-                                        int32_t& y, int32_t& w) {
-  const uint32_t p = in ? __ldg(&arc[k]) : 0u;
-  y = (int32_t)(AM == AM_UNIT ? p : p & ((1u << a.cb) - 1u));
-  w = AM == AM_UNIT ? 1 : (int32_t)(p >> a.cb);
-}
+// One round of a warp's walk: 32 * ILP arcs.
+template <int ILP>
+struct SrcRound {
+  uint32_t p[ILP];                     // the arcs' words
+  uint32_t t;                          // their rows' places in the batch, 8 bits each
+  __device__ __forceinline__ int row(int r) const { return (int)((t >> (8 * r)) & 31u); }
+};
 
 // The rows of a batch: lane i holds row i (first arc, length; 0 when it has
 // none to walk).  Rows of SRC_BIG_ARCS arcs and more are walked one after the
 // other by the whole warp, the others as one flat list of arcs found by a
 // search over the lengths' prefix sums, so that short rows still fill the
-// lanes.  f(place, far end, weight, valid) is called by the whole warp, ILP
-// times in a row after the arcs of all of them were loaded; g() after each such
-// round.
-template <int AM, int ILP, class F, class G>
-__device__ __forceinline__ void src_walk(const SrcArgs& a, const uint32_t* __restrict__ arc, int64_t beg, int32_t len,
-                                         F f, G g) {
+// lanes.  f(round, left) is called by the whole warp; lane l's arc r is there
+// when 32 r + l < left (left is a constant for whole rounds of big rows).
+template <int ILP, class F>
+__device__ __forceinline__ void src_walk(const uint32_t* __restrict__ arc, int64_t beg, int32_t len, F f) {
   const unsigned lane = lane_id();
+  SrcRound<ILP> x;
   uint32_t big = __ballot_sync(0xffffffffu, len >= SRC_BIG_ARCS);
   while (big) {
     const int t = __ffs(big) - 1;
     big &= big - 1;
-    const int64_t b = __shfl_sync(0xffffffffu, beg, t);
+    const uint32_t* a0 = arc + __shfl_sync(0xffffffffu, beg, t) + lane;
     const int32_t n = __shfl_sync(0xffffffffu, len, t);
-    for (int32_t k = (int32_t)lane; k - (int32_t)lane < n; k += 32 * ILP) {
-      int32_t y[ILP], w[ILP];
+    x.t = (uint32_t)t * 0x01010101u;
+    int32_t k = 0;
+    for (; k + 32 * ILP <= n; k += 32 * ILP) {
 #pragma unroll
-      for (int r = 0; r < ILP; r++) src_arc<AM>(a, arc, b + k + 32 * r, k + 32 * r < n, y[r], w[r]);
-      f(y, w, [&](int) { return t; }, [&](int r) { return k + 32 * r < n; });
-      g();
+      for (int r = 0; r < ILP; r++) x.p[r] = __ldg(a0 + k + 32 * r);
+      f(x, std::integral_constant<int, 32 * ILP>());
+    }
+    if (k < n) {
+#pragma unroll
+      for (int r = 0; r < ILP; r++) x.p[r] = k + 32 * r + (int32_t)lane < n ? __ldg(a0 + k + 32 * r) : 0u;
+      f(x, n - k);
     }
   }
   const int32_t sl = len < SRC_BIG_ARCS ? len : 0;
@@ -259,28 +301,22 @@ __device__ __forceinline__ void src_walk(const SrcArgs& a, const uint32_t* __res
   const int32_t excl = incl - sl;
   const int32_t T = __shfl_sync(0xffffffffu, incl, 31);
   for (int32_t p0 = 0; p0 < T; p0 += 32 * ILP) {
-    int32_t y[ILP], w[ILP];
-    int t[ILP];
+    x.t = 0u;
 #pragma unroll
     for (int r = 0; r < ILP; r++) {
       const int32_t p = p0 + 32 * r + (int32_t)lane;
-      t[r] = 0;
-      if (p0 + 32 * r < T) {                             // (uniform)
+      x.p[r] = 0u;
+      if (p0 + 32 * r >= T) continue;                    // (uniform)
+      int t = 0;
 #pragma unroll
-        for (int step = 16; step; step >>= 1) {          // largest t with excl_t <= p
-          const int32_t e = __shfl_sync(0xffffffffu, excl, t[r] + step);
-          if (e <= p) t[r] += step;
-        }
-        const int32_t e = __shfl_sync(0xffffffffu, excl, t[r]);
-        const int64_t b = __shfl_sync(0xffffffffu, beg, t[r]);
-        src_arc<AM>(a, arc, b + (p - e), p < T, y[r], w[r]);
-      } else {
-        y[r] = 0;
-        w[r] = 1;
-      }
+      for (int step = 16; step; step >>= 1)              // the last row that starts at or before p
+        if (__shfl_sync(0xffffffffu, excl, t + step) <= p) t += step;
+      const int32_t e = __shfl_sync(0xffffffffu, excl, t);
+      const int64_t b = __shfl_sync(0xffffffffu, beg, t);
+      if (p < T) x.p[r] = __ldg(arc + (b + (p - e)));
+      x.t |= (uint32_t)t << (8 * r);
     }
-    f(y, w, [&](int r) { return t[r]; }, [&](int r) { return p0 + 32 * r + (int32_t)lane < T; });
-    g();
+    f(x, T - p0);
   }
 }
 
@@ -294,15 +330,18 @@ struct SrcCtx {
   int32_t mv;                          // this lane's vertex of the batch
   unsigned long long nbytes;
 
+  __device__ __forceinline__ int32_t head(uint32_t p) const {
+    return (int32_t)(AM == AM_UNIT ? p : p & ((1u << a.cb) - 1u));
+  }
+  __device__ __forceinline__ int32_t weight(uint32_t p) const { return AM == AM_UNIT ? 1 : (int32_t)(p >> a.cb); }
   template <class Sum, bool COUNT>
   __device__ __forceinline__ void drain(bool all) {
     if (qn < 32 && !(all && qn)) return;
     __syncwarp();
     int q = 0;
-    constexpr bool RECORD = COUNT && !UNIT;
-    while (qn - q >= 32) { src_flush<Sum, COUNT, RECORD>(a, wb, st, q, 32, mv); q += 32; }
+    while (qn - q >= 32) { src_flush<Sum, COUNT>(a, wb, st, q, 32, mv); q += 32; }
     if (all) {
-      if (qn - q) src_flush<Sum, COUNT, RECORD>(a, wb, st, q, qn - q, mv);
+      if (qn - q) src_flush<Sum, COUNT>(a, wb, st, q, qn - q, mv);
       qn = 0;
       return;
     }
@@ -331,10 +370,9 @@ struct SrcCtx {
   // Entries past the bucket's room are not stored: the count tells the step to
   // look through all distances instead.
   __device__ __forceinline__ void offer(int32_t y, int32_t w, int32_t cand, int slot) {
-    if (!st.lower(y, cand)) return;
     if (UNIT) {
-      st.order[atomicAdd(&st.sh.tail, 1u)] = y;
-    } else {
+      if (st.claim(y, cand)) st.order[atomicAdd(&st.sh.tail, 1u)] = y;
+    } else if (st.lower(y, cand)) {
       int b = slot + w;
       if (b >= a.B) b -= a.B;
       const uint32_t at = atomicAdd(&st.cnt[b], 1u);
@@ -347,62 +385,79 @@ struct SrcCtx {
   template <bool PULL, bool PUSH, class Sum>
   __device__ __forceinline__ void fwd(const uint32_t* arc, int64_t beg, int32_t len, int32_t d, int slot) {
     if (a.bytes) nbytes += 8ull * (unsigned long long)len;
-    src_walk<AM, ILP>(a, arc, beg, len,
-        [&](const int32_t (&y)[ILP], const int32_t (&w)[ILP], auto place, auto valid) {
-          int32_t dy[ILP];
+    src_walk<ILP>(arc, beg, len, [&](const SrcRound<ILP>& x, auto left) {
+      int32_t dy[ILP];
+      bool tight = false, nearer = false;
 #pragma unroll
-          for (int r = 0; r < ILP; r++) dy[r] = valid(r) ? st.tau(y[r]) : d;      // d: neither tight nor improved
+      for (int r = 0; r < ILP; r++) {                   // -2: neither tight nor improved
+        dy[r] = 32 * r + (int)lane_id() < left ? (int32_t)st.dist[head(x.p[r])] : -2;
+        tight |= dy[r] + weight(x.p[r]) == d;           // (unreached entries pass no test, see redo)
+        nearer |= d + weight(x.p[r]) < dy[r];
+      }
+      if (PULL && __any_sync(0xffffffffu, tight)) {
 #pragma unroll
-          for (int r = 0; r < ILP; r++) {
-            if (PULL) list(dy[r] < d && dy[r] + w[r] == d, y[r], place(r));
-            if (PUSH && d + w[r] < dy[r]) offer(y[r], w[r], d + w[r], slot);
-          }
-        },
-        [&]() { if (PULL) drain<Sum, true>(false); });
+        for (int r = 0; r < ILP; r++) list(dy[r] + weight(x.p[r]) == d, head(x.p[r]), x.row(r));
+      }
+      if (PUSH && nearer) {
+#pragma unroll
+        for (int r = 0; r < ILP; r++)
+          if (d + weight(x.p[r]) < dy[r]) offer(head(x.p[r]), weight(x.p[r]), d + weight(x.p[r]), slot);
+      }
+      if (PULL) {
+        __syncwarp();
+        drain<Sum, true>(false);
+      }
+    });
   }
   // MFBr rows: this lane's vertex is at distance d.
   template <class Sum>
   __device__ __forceinline__ void bwd(int64_t beg, int32_t len, int32_t d) {
     if (a.bytes) nbytes += 8ull * (unsigned long long)len;
-    src_walk<AM, ILP>(a, a.arc, beg, len,
-        [&](const int32_t (&y)[ILP], const int32_t (&w)[ILP], auto place, auto valid) {
-          int32_t dy[ILP];
+    src_walk<ILP>(a.arc, beg, len, [&](const SrcRound<ILP>& x, auto left) {
+      int32_t dy[ILP];
 #pragma unroll
-          for (int r = 0; r < ILP; r++) dy[r] = valid(r) ? st.tau(y[r]) : -1;
+      for (int r = 0; r < ILP; r++) dy[r] = 32 * r + (int)lane_id() < left ? st.tau(head(x.p[r])) : -1;
 #pragma unroll
-          for (int r = 0; r < ILP; r++) {
-            const int32_t dv = __shfl_sync(0xffffffffu, d, place(r));
-            list(dy[r] == dv + w[r], y[r], place(r));
-          }
-        },
-        [&]() { drain<Sum, false>(false); });
+      for (int r = 0; r < ILP; r++) {
+        const int32_t dv = __shfl_sync(0xffffffffu, d, x.row(r));
+        list(dy[r] == dv + weight(x.p[r]), head(x.p[r]), x.row(r));
+      }
+      drain<Sum, false>(false);
+    });
   }
 };
 
-// sigma_bar of a settled vertex: stored, and checked against 2^53 (FP64
-// output inexact) and, for 64-bit counts, 2^58 (later sums could wrap: the
-// source is redone in FP64).
-__device__ __forceinline__ void src_put_count(const SrcArgs& a, SrcShared& sh, uint64_t* slot, const SumF64& x) {
-  *slot = x.bits();
+// sigma_bar as FP64.
+template <bool UNIT>
+__device__ __forceinline__ double src_sigma(uint64_t sv) {
+  return UNIT ? (double)sv : __longlong_as_double((long long)sv);
+}
+// sigma_bar of a settled vertex: stored beside a zeta of 0, and checked against
+// 2^53 (FP64 output inexact) and, for 64-bit counts, 2^58 (later sums could
+// wrap: the source is redone in FP64).
+__device__ __forceinline__ void src_put(SrcCell* c, uint64_t sv) {
+  *reinterpret_cast<ulonglong2*>(c) = make_ulonglong2(sv, 0ull);
+}
+template <class S>
+__device__ __forceinline__ void src_put_count(const SrcArgs& a, S& st, int32_t v, const SumF64& x) {
+  src_put(&st.cell[v], x.bits());
   if (x.s >= 9007199254740992.0) atomicOr(&a.ctl->flags, FLAG_SIGMA_INEXACT);
 }
-__device__ __forceinline__ void src_put_count(const SrcArgs& a, SrcShared& sh, uint64_t* slot, const SumU64& x) {
-  *slot = x.i;
+template <class S>
+__device__ __forceinline__ void src_put_count(const SrcArgs& a, S& st, int32_t v, const SumU64& x) {
+  src_put(&st.cell[v], x.i);
   if (x.i >= (1ull << 53)) {
     atomicOr(&a.ctl->flags, FLAG_SIGMA_INEXACT);
-    if (x.i >= (1ull << 58)) sh.redo = 1u;
+    if (x.i >= (1ull << 58)) st.sh.redo = 1u;
   }
 }
-// zeta of a vertex: its lambda term, and the value zeta + 1/sigma_bar.
-__device__ __forceinline__ void src_put_value(uint64_t* slot, double* lam, const SumF64& x) {
-  const double sg = __longlong_as_double((long long)*slot);
+// zeta of a vertex (pulled form): its lambda term, and the value zeta +
+// 1/sigma_bar in the place of the count.
+template <bool UNIT>
+__device__ __forceinline__ void src_put_value(SrcCell* c, double* lam, const SumF64& x) {
+  const double sg = src_sigma<UNIT>(c->sv);
   if (x.s != 0.0) atomicAdd(lam, x.s * sg);
-  *slot = (uint64_t)__double_as_longlong(x.s + 1.0 / sg);
-}
-__device__ __forceinline__ void src_put_value(uint64_t* slot, double* lam, const SumDF& x) {
-  float ls = 0.f, lc = 0.f;
-  *slot = finish_col(acc_value(x.s, x.c), *slot, ls, lc);
-  if (ls != 0.f) atomicAdd(lam, (double)ls + (double)lc);
+  c->sv = (uint64_t)__double_as_longlong(x.s + 1.0 / sg);
 }
 
 // Hub rows: a warp's share of the row's sum joins the total; the total read back.
@@ -410,16 +465,8 @@ __device__ __forceinline__ void src_hub_add(SrcShared& sh, int h, const SumF64& 
 __device__ __forceinline__ void src_hub_add(SrcShared& sh, int h, const SumU64& x) {
   atomicAdd(&sh.hcnt[h], (unsigned long long)x.i);
 }
-__device__ __forceinline__ void src_hub_add(SrcShared& sh, int h, const SumDF& x) {
-  atomicAdd(&sh.hacc[h], (double)x.s + (double)x.c);
-}
 __device__ __forceinline__ void src_hub_get(const SrcShared& sh, int h, SumF64& x) { x.s = sh.hacc[h]; }
 __device__ __forceinline__ void src_hub_get(const SrcShared& sh, int h, SumU64& x) { x.i = sh.hcnt[h]; }
-__device__ __forceinline__ void src_hub_get(const SrcShared& sh, int h, SumDF& x) {
-  const dfl v = df_of_double(sh.hacc[h]);
-  x.s = v.hi;
-  x.c = v.lo;
-}
 // Lists v as a hub row of the step, cut into `pieces`; false when the list is
 // full.  One atomic gives the place and the first piece, so both grow together.
 __device__ __forceinline__ bool src_list_hub(SrcShared& sh, int32_t v, uint32_t pieces) {
@@ -450,19 +497,19 @@ __device__ __forceinline__ uint32_t src_batch(uint32_t items, int nwarp) {
   return bs;
 }
 
-// UNIT: unit weights, 64-bit counts and double-float values; otherwise FP64.
-// SSV: sv in shared memory.  SYM: undirected.
-template <bool UNIT, int DM, bool SSV, int AM, bool SYM>
+// UNIT: unit weights by levels, 64-bit counts; otherwise integer weights (or
+// none, AM_UNIT) by distance, FP64 counts.  SYM: undirected.
+template <bool UNIT, int DM, int AM, bool SYM>
 __global__ void __launch_bounds__(1024) k_src_bc(SrcArgs a) {
-  constexpr int ILP = SSV ? 2 : 4;
+  constexpr int ILP = 4;
   using Cnt = typename std::conditional<UNIT, SumU64, SumF64>::type;
-  using Val = typename std::conditional<UNIT, SumDF, SumF64>::type;
+  using Val = SumF64;
   using D = typename SrcState<DM>::D;
   extern __shared__ __align__(16) unsigned char src_raw[];
   SrcShared& sh = *reinterpret_cast<SrcShared*>(src_raw);
   char* slot_mem = a.slots + (size_t)blockIdx.x * a.slot_bytes;
   const int wid = (int)threadIdx.x >> 5, nwarp = (int)blockDim.x >> 5;
-  const size_t n8 = ((size_t)a.n + 7) & ~size_t(7);
+  const size_t n8 = ((size_t)a.n + 15) & ~size_t(15);
   unsigned char* sp = src_raw + src_al16(sizeof(SrcShared));
   SrcWarp<ILP>& wb = reinterpret_cast<SrcWarp<ILP>*>(sp)[wid];
   sp += src_al16(sizeof(SrcWarp<ILP>) * nwarp);
@@ -470,15 +517,13 @@ __global__ void __launch_bounds__(1024) k_src_bc(SrcArgs a) {
   if (!UNIT) sp += src_al16((size_t)a.B * 4);
   int32_t* s_ring = reinterpret_cast<int32_t*>(sp);
   if (!UNIT) sp += src_al16((size_t)a.B * a.scap * 4);
-  uint64_t* s_sv = reinterpret_cast<uint64_t*>(sp);
-  if (SSV) sp += 8 * n8;
-  D* s_dist = reinterpret_cast<D*>(sp);
-  if (DM != DM_GLOBAL) sp += sizeof(D) * n8;
-  int32_t* order = a.so ? reinterpret_cast<int32_t*>(sp) : reinterpret_cast<int32_t*>(slot_mem + a.o_order);
-  SrcState<DM> st{sh, s_cnt, s_ring, DM != DM_GLOBAL ? s_dist : reinterpret_cast<D*>(slot_mem + a.o_dist),
-                  SSV ? s_sv : reinterpret_cast<uint64_t*>(slot_mem + a.o_sv), order,
-                  reinterpret_cast<uint32_t*>(order + n8), reinterpret_cast<int32_t*>(slot_mem + a.o_ring),
-                  reinterpret_cast<double*>(slot_mem + a.o_z), reinterpret_cast<int2*>(slot_mem + a.o_dag)};
+  SrcState<DM> st{sh, s_cnt, s_ring,
+                  DM != DM_GLOBAL ? reinterpret_cast<D*>(sp) : reinterpret_cast<D*>(slot_mem + a.o_dist),
+                  reinterpret_cast<SrcCell*>(slot_mem + a.o_cell),
+                  reinterpret_cast<int32_t*>(slot_mem + a.o_order),
+                  reinterpret_cast<uint2*>(slot_mem + a.o_order + 4 * n8),
+                  reinterpret_cast<int32_t*>(slot_mem + a.o_ring),
+                  reinterpret_cast<uint32_t*>(slot_mem + a.o_dag), a.n <= 65536};
   SrcCtx<UNIT, DM, AM, ILP> cx{a, st, wb, 0, 0, 0ull};
   const unsigned lane = lane_id();
   const uint32_t lt = (1u << lane) - 1u;
@@ -499,8 +544,8 @@ __global__ void __launch_bounds__(1024) k_src_bc(SrcArgs a) {
       if (threadIdx.x == 0) atomicOr(&a.ctl->flags, FLAG_BAD_SOURCE);
       continue;
     }
-    if (DM == DM_SMEM16) {
-      for (uint32_t i = threadIdx.x; i < (uint32_t)(n8 / 8); i += blockDim.x)
+    if (DM == DM_SMEM16 || DM == DM_SMEM8) {
+      for (uint32_t i = threadIdx.x; i < (uint32_t)(n8 * sizeof(D) / 16); i += blockDim.x)
         reinterpret_cast<uint4*>(st.dist)[i] = make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu);
     } else {
       for (int32_t v = (int32_t)threadIdx.x; v < a.n; v += (int32_t)blockDim.x) st.dist[v] = (D)INF;
@@ -510,8 +555,7 @@ __global__ void __launch_bounds__(1024) k_src_bc(SrcArgs a) {
     __syncthreads();
     if (threadIdx.x == 0) {
       st.dist[s] = 0;
-      st.off[0] = 0u;
-      if (!UNIT) st.off[1] = 0u;
+      st.off[0] = make_uint2(0u, 0u);
       if (UNIT) st.order[0] = s;
       else {
         st.cnt[0] = 1u;
@@ -584,10 +628,7 @@ __global__ void __launch_bounds__(1024) k_src_bc(SrcArgs a) {
         }
         cx.template drain<Cnt, true>(true);
         __syncwarp();
-        if (mine) {
-          src_put_count(a, sh, &st.sv[v], Cnt::of_count(d == 0 ? Cnt::one() : wb.acc[lane]));
-          if (!UNIT) st.z[v] = 0.0;
-        }
+        if (mine) src_put_count(a, st, v, Cnt::of_count(d == 0 ? Cnt::one() : wb.acc[lane]));
         __syncwarp();
       }
       const bool hubs = __syncthreads_or(hub);          // the same answer for every thread
@@ -622,8 +663,7 @@ __global__ void __launch_bounds__(1024) k_src_bc(SrcArgs a) {
         for (uint32_t h = threadIdx.x; h < nh; h += blockDim.x) {
           Cnt x;
           src_hub_get(sh, (int)h, x);
-          if (!UNIT) st.z[sh.hv[h]] = 0.0;
-          src_put_count(a, sh, &st.sv[sh.hv[h]], d == 0 ? Cnt::of_count(Cnt::one()) : x);
+          src_put_count(a, st, sh.hv[h], d == 0 ? Cnt::of_count(Cnt::one()) : x);
         }
         if (threadIdx.x == 0) sh.nhub = 0ull;
       }
@@ -631,9 +671,10 @@ __global__ void __launch_bounds__(1024) k_src_bc(SrcArgs a) {
         if (hubs) __syncthreads();                      // the hubs' sums are stored
         q0 = q1;
         q1 = sh.tail;
-        redo = sh.redo != 0u;
+        // (a count past 2^58, or a level past which a narrow tau cannot go)
+        redo = sh.redo != 0u || (DM != DM_GLOBAL && d + 2 >= SrcState<DM>::NONE);
         k++;
-        if (threadIdx.x == 0) st.off[k] = q0;
+        if (threadIdx.x == 0) st.off[k] = make_uint2(q0, sh.dtail);
         __syncthreads();                                // every thread has read tail and redo
         d++;
         if (q1 == q0 || redo) break;
@@ -649,13 +690,13 @@ __global__ void __launch_bounds__(1024) k_src_bc(SrcArgs a) {
             if (bal) { nd = d + j0 + __ffs(bal) - 1; break; }
           }
           if (lane == 0) {
-            sh.next = DM == DM_SMEM16 && sh.redo ? -1 : nd;
+            // distances of the next step's offers must stay below an unreached entry's
+            if (DM == DM_SMEM16 && nd >= SrcState<DM>::NONE - a.B) { sh.redo = 1u; nd = -1; }
+            sh.next = nd;
             st.cnt[slot] = 0u;
             if (sh.tail != sh.mark) {                   // a step of stale entries settles nothing
               sh.mark = sh.tail;
-              const uint32_t t = ++sh.steps;
-              st.off[2 * t] = sh.tail;
-              st.off[2 * t + 1] = sh.dtail;
+              st.off[++sh.steps] = make_uint2(sh.tail, sh.dtail);
             }
           }
         }
@@ -683,36 +724,46 @@ __global__ void __launch_bounds__(1024) k_src_bc(SrcArgs a) {
         a.dist_out[(size_t)si * a.n + v] = x;
         if (a.sigma_out)
           a.sigma_out[(size_t)si * a.n + v] =
-              x == INF ? 0.0 : (UNIT ? (double)st.sv[v] : __longlong_as_double((long long)st.sv[v]));
+              x == INF ? 0.0 : src_sigma<UNIT>(st.cell[v].sv);
       }
     }
     if (!a.lambda) continue;
     // ---- MFBr: the same steps backwards (step 0 is the source)
     double* lam = a.lambda + (a.row ? (size_t)a.row[si] * a.n : 0);
-    if (!UNIT && sh.dtail <= a.dcap) {
+    if (sh.dtail <= a.dcap) {
       // over the recorded DAG arcs (v, u): zeta(u) += zeta(v) + 1/sigma_bar(v).
       // Only zeta(v) depends on the step before, so a step's first arcs and
       // their 1/sigma_bar are loaded one step ahead.
       const uint32_t tid = threadIdx.x, T = blockDim.x;
-      uint32_t e1 = st.off[2 * k + 1], e0 = st.off[2 * k - 1], em = k > 1 ? st.off[2 * k - 3] : 0u;
+      uint32_t e1 = st.off[k].y, e0 = st.off[k - 1].y, em = k > 1 ? st.off[k - 2].y : 0u;
       int2 cur = make_int2(s, s);
       double rs = 0.0;
       if (e0 + tid < e1) {
-        cur = st.dag[e0 + tid];
-        rs = 1.0 / __longlong_as_double((long long)st.sv[cur.x]);
+        cur = st.arc(e0 + tid);
+        rs = 1.0 / src_sigma<UNIT>(st.cell[cur.x].sv);
       }
       for (uint32_t t = k; t-- > 1;) {
-        const uint32_t en = t > 1 ? st.off[2 * t - 3] : 0u;
+        const uint32_t en = t > 1 ? st.off[t - 2].y : 0u;
         int2 nxt = make_int2(s, s);
         double nrs = 0.0;
-        if (t > 1 && em + tid < e0) nxt = st.dag[em + tid];
-        if (cur.y != s) atomicAdd(&st.z[cur.y], __ldcg(&st.z[cur.x]) + rs);
-        for (uint32_t e = e0 + tid + T; e < e1; e += T) {
-          const int2 x = st.dag[e];
-          if (x.y != s)
-            atomicAdd(&st.z[x.y], __ldcg(&st.z[x.x]) + 1.0 / __longlong_as_double((long long)st.sv[x.x]));
+        if (t > 1 && em + tid < e0) nxt = st.arc(em + tid);
+        if (cur.y != s) atomicAdd(&st.cell[cur.y].z, __ldcg(&st.cell[cur.x].z) + rs);
+        for (uint32_t e = e0 + tid + T; e < e1; e += ILP * T) {
+          int2 x[ILP];
+          double z[ILP], sg[ILP];
+#pragma unroll
+          for (int r = 0; r < ILP; r++) x[r] = e + r * T < e1 ? st.arc(e + r * T) : make_int2(s, s);
+#pragma unroll
+          for (int r = 0; r < ILP; r++)
+            if (x[r].y != s) {
+              z[r] = __ldcg(&st.cell[x[r].x].z);
+              sg[r] = src_sigma<UNIT>(st.cell[x[r].x].sv);
+            }
+#pragma unroll
+          for (int r = 0; r < ILP; r++)
+            if (x[r].y != s) atomicAdd(&st.cell[x[r].y].z, z[r] + 1.0 / sg[r]);
         }
-        if (nxt.y != s) nrs = 1.0 / __longlong_as_double((long long)st.sv[nxt.x]);
+        if (nxt.y != s) nrs = 1.0 / src_sigma<UNIT>(st.cell[nxt.x].sv);
         if (a.bytes) cx.nbytes += e0 + tid < e1 ? 32ull * ((e1 - e0 - tid + T - 1) / T) : 0ull;
         __syncthreads();
         e1 = e0;
@@ -721,18 +772,26 @@ __global__ void __launch_bounds__(1024) k_src_bc(SrcArgs a) {
         cur = nxt;
         rs = nrs;
       }
-      for (uint32_t i = 1 + tid; i < sh.tail; i += T) {        // (entry 0 is the source)
-        const int32_t v = st.order[i];
-        const double z = __ldcg(&st.z[v]);
-        if (z != 0.0) atomicAdd(&lam[v], z * __longlong_as_double((long long)st.sv[v]));
-        if (a.bytes) cx.nbytes += 28;
+      for (uint32_t i = 1 + tid; i < sh.tail; i += ILP * T) {  // (entry 0 is the source)
+        int32_t v[ILP];
+        double z[ILP], sg[ILP];
+#pragma unroll
+        for (int r = 0; r < ILP; r++) v[r] = i + r * T < sh.tail ? st.order[i + r * T] : -1;
+#pragma unroll
+        for (int r = 0; r < ILP; r++) {
+          z[r] = v[r] >= 0 ? __ldcg(&st.cell[v[r]].z) : 0.0;
+          sg[r] = v[r] >= 0 ? src_sigma<UNIT>(st.cell[v[r]].sv) : 0.0;
+        }
+#pragma unroll
+        for (int r = 0; r < ILP; r++)
+          if (z[r] != 0.0) atomicAdd(&lam[v[r]], z[r] * sg[r]);
       }
+      if (a.bytes && tid == 0) cx.nbytes += 28ull * sh.tail;
       continue;
     }
-    // (unit weights, or more DAG arcs than recorded: pulled over the out-arcs)
-    constexpr int OS = UNIT ? 1 : 2;                    // stride of off
+    // more DAG arcs than recorded: pulled over the out-arcs
     for (uint32_t t = k; t-- > 1;) {
-      const uint32_t o0 = st.off[OS * t], items = st.off[OS * (t + 1)] - o0;
+      const uint32_t o0 = st.off[t].x, items = st.off[t + 1].x - o0;
       const uint32_t bs = src_batch(items, nwarp);
       bool hub = false;
       for (uint32_t i0 = (uint32_t)wid * bs; i0 < items; i0 += (uint32_t)nwarp * bs) {
@@ -757,7 +816,7 @@ __global__ void __launch_bounds__(1024) k_src_bc(SrcArgs a) {
         cx.template bwd<Val>(b, len, dv);
         cx.template drain<Val, false>(true);
         __syncwarp();
-        if (mine) src_put_value(&st.sv[v], &lam[v], Val::of_value(wb.acc[lane]));
+        if (mine) src_put_value<UNIT>(&st.cell[v], &lam[v], Val::of_value(wb.acc[lane]));
         if (a.bytes && mine) cx.nbytes += 24;
         __syncwarp();
       }
@@ -782,7 +841,7 @@ __global__ void __launch_bounds__(1024) k_src_bc(SrcArgs a) {
         for (uint32_t h = threadIdx.x; h < nh; h += blockDim.x) {
           Val x;
           src_hub_get(sh, (int)h, x);
-          src_put_value(&st.sv[sh.hv[h]], &lam[sh.hv[h]], x);
+          src_put_value<UNIT>(&st.cell[sh.hv[h]], &lam[sh.hv[h]], x);
         }
         if (threadIdx.x == 0) sh.nhub = 0ull;
         __syncthreads();
@@ -797,17 +856,20 @@ __global__ void __launch_bounds__(1024) k_src_bc(SrcArgs a) {
 }
 
 // ------------------------------------------------------------------ driver
-template <bool UNIT, int DM, bool SSV, int AM>
+template <bool UNIT, int DM, int AM>
 static const void* src_pick(bool sym) {
-  return sym ? (const void*)k_src_bc<UNIT, DM, SSV, AM, true> : (const void*)k_src_bc<UNIT, DM, SSV, AM, false>;
+  return sym ? (const void*)k_src_bc<UNIT, DM, AM, true> : (const void*)k_src_bc<UNIT, DM, AM, false>;
 }
 static const void* src_kernel(const SourcePlan& p, bool sym) {
-  if (p.am == AM_PACKED) {
-    if (p.dm == DM_SMEM16) return src_pick<false, DM_SMEM16, false, AM_PACKED>(sym);
-    if (p.dm == DM_SMEM32) return src_pick<false, DM_SMEM32, false, AM_PACKED>(sym);
-    return src_pick<false, DM_GLOBAL, false, AM_PACKED>(sym);
+  if (p.unit) {
+    if (p.dm == DM_SMEM16) return src_pick<true, DM_SMEM16, AM_UNIT>(sym);
+    if (p.dm == DM_SMEM8) return src_pick<true, DM_SMEM8, AM_UNIT>(sym);
+    return src_pick<true, DM_GLOBAL, AM_UNIT>(sym);
   }
-  return src_pick<false, DM_GLOBAL, false, AM_UNIT>(sym);
+  if (p.am == AM_UNIT) return src_pick<false, DM_GLOBAL, AM_UNIT>(sym);
+  if (p.dm == DM_SMEM16) return src_pick<false, DM_SMEM16, AM_PACKED>(sym);
+  if (p.dm == DM_SMEM32) return src_pick<false, DM_SMEM32, AM_PACKED>(sym);
+  return src_pick<false, DM_GLOBAL, AM_PACKED>(sym);
 }
 
 static int pow2_floor(int64_t x) {
@@ -816,16 +878,37 @@ static int pow2_floor(int64_t x) {
   return p;
 }
 
-// wide: distances in 32 bits, the form that sources are redone in.
-void source_plan(const DevGraph& g, int cols, bool wide, SourcePlan& p) {
+// unit: by levels, 64-bit counts.  wide: FP64 counts and distances in 32 bits,
+// the form that sources are redone in.
+void source_plan(const DevGraph& g, int cols, bool unit, bool wide, SourcePlan& p) {
   const int64_t n = std::max(g.n, 1);
-  const int64_t n8 = (n + 7) & ~int64_t(7);
+  const int64_t n8 = (n + 15) & ~int64_t(15);
   const int64_t avg = g.nnz / n;
-  const int64_t per_sm = std::max<int64_t>(1, (cols + SRC_SMS - 1) / SRC_SMS);   // sources an SM should hold
+  int64_t per_sm = std::max<int64_t>(1, (cols + SRC_SMS - 1) / SRC_SMS);         // sources an SM should hold
   p = SourcePlan{};
-  p.B = g.wmax + 1;
+  p.unit = unit && !wide;
+  p.B = p.unit ? 0 : g.wmax + 1;
   p.am = g.w ? AM_PACKED : AM_UNIT;
-  p.scap = (uint32_t)std::min<int64_t>(64, 8192 / (4 * p.B));
+  p.scap = p.unit ? 0u : (uint32_t)std::min<int64_t>(64, 8192 / (4 * p.B));
+  if (!p.unit) {
+    p.cap = (uint32_t)std::min<int64_t>(n, std::max<int64_t>(512, std::min<int64_t>(n / 8, 16 * n / p.B)));
+    p.cap = std::max(p.cap, p.scap + 1);
+  }
+  // DAG arcs for MFBr: all there can be (an undirected edge is one in at most
+  // one direction), or 32 per vertex; sources with more pull instead
+  p.dcap = (uint32_t)std::min<int64_t>(g.directed ? g.nnz : g.nnz / 2, 32 * n8);
+  auto layout = [&](bool tau) {
+    Carver c(nullptr, 0);
+    p.o_cell = c.off; c.take<ulonglong2>((size_t)n8);    // (SrcCell)
+    p.o_dist = c.off; c.take<int32_t>(tau ? (size_t)n8 : 0);
+    p.o_order = c.off; c.take<int32_t>((size_t)(3 * n8 + 16));
+    p.o_ring = c.off; c.take<int32_t>((size_t)p.B * (p.cap - p.scap));
+    p.o_dag = c.off; c.take<uint32_t>((size_t)p.dcap * (n <= 65536 ? 1 : 2));
+    return c.off;
+  };
+  // unit-weight graphs: at most 256 MB of block states, but two sources an SM
+  if (p.unit)
+    per_sm = std::min(per_sm, std::max<int64_t>(2, (256ll << 20) / (int64_t)layout(false) / SRC_SMS));
   const int64_t ring = (int64_t)src_al16((size_t)p.B * 4) + (int64_t)src_al16((size_t)p.B * p.scap * 4);
   auto fixed = [&](int threads) {
     return (int64_t)src_al16(sizeof(SrcShared)) + (int64_t)src_al16(sizeof(SrcWarp<4>) * (threads / 32)) + ring;
@@ -839,9 +922,10 @@ void source_plan(const DevGraph& g, int cols, bool wide, SourcePlan& p) {
   p.dm = DM_GLOBAL;
   p.threads = std::max(g.max_deg, g.max_in_deg) <= 8 ? threads_for(share) : 1024;
   int64_t db = 0;
-  const int form[2] = {DM_SMEM32, DM_SMEM16};
-  for (int f = 0; f < (wide ? 1 : 2) && p.am == AM_PACKED && p.dm == DM_GLOBAL; f++) {
-    const int64_t bytes = f == 0 ? 4 : 2;
+  const int form[2] = {p.unit ? DM_SMEM16 : DM_SMEM32, p.unit ? DM_SMEM8 : DM_SMEM16};
+  const int forms = p.unit ? 2 : p.am != AM_PACKED ? 0 : wide ? 1 : 2;
+  for (int f = 0; f < forms && p.dm == DM_GLOBAL; f++) {
+    const int64_t bytes = (p.unit ? 2 : 4) >> f;
     if (room(threads_for(share), bytes) >= share) {
       p.dm = form[f];
       db = bytes;
@@ -856,22 +940,11 @@ void source_plan(const DevGraph& g, int cols, bool wide, SourcePlan& p) {
     }
   }
   const int64_t smem = fixed(p.threads) + db * n8;
-  const int64_t resident = std::max<int64_t>(1, std::min<int64_t>(room(p.threads, db), 1024 / p.threads));
+  const int64_t resident =
+      std::max<int64_t>(1, std::min({room(p.threads, db), (int64_t)(1024 / p.threads), p.unit ? per_sm : int64_t(8)}));
   p.slots = (int)std::max<int64_t>(1, std::min<int64_t>(cols, SRC_SMS * resident));
   p.smem = (size_t)smem;
-  p.cap = (uint32_t)std::min<int64_t>(n, std::max<int64_t>(512, std::min<int64_t>(n / 8, 16 * n / p.B)));
-  p.cap = std::max(p.cap, p.scap + 1);
-  Carver c(nullptr, 0);
-  p.o_sv = c.off; c.take<uint64_t>((size_t)n8);
-  p.o_dist = c.off; c.take<int32_t>(p.dm == DM_GLOBAL ? (size_t)n8 : 0);
-  p.o_z = c.off; c.take<double>((size_t)n8);
-  p.o_order = c.off; c.take<int32_t>((size_t)(3 * n8 + 16));
-  p.o_ring = c.off; c.take<int32_t>((size_t)p.B * (p.cap - p.scap));
-  // DAG arcs for MFBr: all there can be (an undirected edge is one in at most
-  // one direction), or 32 per vertex; sources with more pull instead
-  p.dcap = (uint32_t)std::min<int64_t>(g.directed ? g.nnz : g.nnz / 2, 32 * n8);
-  p.o_dag = c.off; c.take<int2>((size_t)p.dcap);
-  p.slot_bytes = c.off;
+  p.slot_bytes = layout(p.dm == DM_GLOBAL);
 }
 
 void source_carve(Carver& c, const SourcePlan& p, int32_t nredo, SourceState& s) {
@@ -909,10 +982,9 @@ mfbc_status source_run(RunCtx& rc, const SourcePlan& p, SourceState& s, const in
   a.sigma_out = sigma_out;
   a.slots = s.slots;
   a.slot_bytes = p.slot_bytes;
-  a.o_dist = p.o_dist; a.o_sv = p.o_sv; a.o_z = p.o_z; a.o_order = p.o_order;
+  a.o_dist = p.o_dist; a.o_cell = p.o_cell; a.o_order = p.o_order;
   a.o_ring = p.o_ring; a.o_dag = p.o_dag;
   a.dcap = lambda ? p.dcap : 0u;
-  a.so = 0;
   a.B = p.B;
   a.scap = p.scap;
   a.cap = p.cap;
