@@ -232,6 +232,7 @@ constexpr size_t LVL_SMEM = sizeof(WarpSmem) * LVL_WARPS;
 #define MFBC_GATHER_U 4
 #endif
 constexpr int GATHER_U = MFBC_GATHER_U;      // gather loads in flight per warp
+static_assert(32 % GATHER_U == 0, "a chunk of 32 staged pairs is worked GATHER_U at a time");
 #ifndef MFBC_GATHER_MIN_BLOCKS
 #define MFBC_GATHER_MIN_BLOCKS 4
 #endif
@@ -592,23 +593,9 @@ struct GatherSmem {
   int32_t seg[32];
 };
 
-__device__ __forceinline__ void ld4(const double* p, double& a, double& b, double& c, double& d) {
-  asm volatile("ld.global.nc.v4.f64 {%0,%1,%2,%3}, [%4];" : "=d"(a), "=d"(b), "=d"(c), "=d"(d) : "l"(p));
-}
-__device__ __forceinline__ void ld4_coherent(const double* p, double& a, double& b, double& c, double& d) {
-  asm volatile("ld.global.v4.f64 {%0,%1,%2,%3}, [%4];" : "=d"(a), "=d"(b), "=d"(c), "=d"(d) : "l"(p) : "memory");
-}
-__device__ __forceinline__ void st4(double* p, double a, double b, double c, double d) {
-  asm volatile("st.global.v4.f64 [%0], {%1,%2,%3,%4};" ::"l"(p), "d"(a), "d"(b), "d"(c), "d"(d) : "memory");
-}
-
-// Gather over a group of up to 32 segments (lane k holds segment k's header).
-// The group's pairs are flattened with a warp scan and staged 32 at a time in
-// shared memory; each pair costs every lane one broadcast row read, one mask
-// word read and, when one of its four columns is set, one 32-byte load.
-// FLUSH(k, acc) is called once per segment with pairs, in order, by the whole
-// warp, with the lane's four column sums and the OR of its 4-bit slices.
-template <bool COUNT>
+// Stages pairs p0 .. p0 + 31 of a group's T pairs (lane k holds segment k's
+// header and the prefix sums of the segments' pair counts); lastmask: the pairs
+// that end their segment.
 __device__ __forceinline__ void stage_chunk(const uint4& myseg, int excl, int incl, int T, int p0,
                                             const uint32_t* __restrict__ prow, const uint4* __restrict__ pmask,
                                             GatherSmem& gs, uint32_t* lastmask) {
@@ -626,12 +613,16 @@ __device__ __forceinline__ void stage_chunk(const uint4& myseg, int excl, int in
   const int texcl = __shfl_sync(0xffffffffu, excl, t);
   const int tincl = __shfl_sync(0xffffffffu, incl, t);
   __syncwarp();
+  uint4 m = make_uint4(0u, 0u, 0u, 0u);              // (places past the last pair: nothing to gather)
+  uint32_t row = 0u;
   if (p < T) {
     const uint32_t at = tpb + (uint32_t)(p - texcl);
-    gs.mask[lane] = pmask[at];
-    gs.row[lane] = prow[at];
-    gs.seg[lane] = t;
+    m = pmask[at];
+    row = prow[at];
   }
+  gs.mask[lane] = m;
+  gs.row[lane] = row;
+  gs.seg[lane] = t;
   *lastmask = __ballot_sync(0xffffffffu, p < T && p + 1 == tincl);
   __syncwarp();
 }
@@ -650,23 +641,41 @@ __device__ __forceinline__ void stage_chunk(const uint4& myseg, int excl, int in
 #ifndef MFBC_GATHER_NC
 #define MFBC_GATHER_NC 0
 #endif
-// Rows of high-degree vertices (bit 31 of the pair's row index) are loaded
-// with the L2 evict-last priority: most DAG arcs end there, so their sectors
-// are read again and again within a level, while the rows of the many
-// low-degree vertices stream through.  A hint only; results do not depend on it.
-#ifndef MFBC_HOT_HINT
-#define MFBC_HOT_HINT 1
-#endif
-__device__ __forceinline__ void ld4u_keep(const uint64_t* p, uint64_t& a, uint64_t& b, uint64_t& c, uint64_t& d) {
-  asm volatile("ld.global.L1::no_allocate.L2::evict_last.v4.u64 {%0,%1,%2,%3}, [%4];"
-               : "=l"(a), "=l"(b), "=l"(c), "=l"(d) : "l"(p));
-}
-__device__ __forceinline__ void ld4u(const uint64_t* p, uint64_t& a, uint64_t& b, uint64_t& c, uint64_t& d) {
+//
+// The load is predicated on the lane's slice sl of the mask; without it the
+// outputs keep whatever the registers held, and nothing of them is added.  (As
+// an ordinary conditional load with zeros otherwise, the gather took 78
+// instructions a pair; with the predicate, the unconditional staging and the
+// common path below it takes 45.)
+__device__ __forceinline__ void ld4u_if(uint32_t sl, const uint64_t* p, uint64_t& a, uint64_t& b, uint64_t& c,
+                                        uint64_t& d) {
 #if MFBC_GATHER_NC
-  asm volatile("ld.global.nc.L1::no_allocate.v4.u64 {%0,%1,%2,%3}, [%4];" : "=l"(a), "=l"(b), "=l"(c), "=l"(d) : "l"(p));
+  asm volatile("{.reg .pred p; setp.ne.u32 p, %5, 0; @p ld.global.nc.L1::no_allocate.v4.u64 {%0,%1,%2,%3}, [%4];}"
+               : "=l"(a), "=l"(b), "=l"(c), "=l"(d) : "l"(p), "r"(sl));
 #else
-  asm volatile("ld.global.L1::no_allocate.v4.u64 {%0,%1,%2,%3}, [%4];" : "=l"(a), "=l"(b), "=l"(c), "=l"(d) : "l"(p));
+  asm volatile("{.reg .pred p; setp.ne.u32 p, %5, 0; @p ld.global.L1::no_allocate.v4.u64 {%0,%1,%2,%3}, [%4];}"
+               : "=l"(a), "=l"(b), "=l"(c), "=l"(d) : "l"(p), "r"(sl));
 #endif
+}
+// L2 priorities of the MFBr gather on large graphs: rows of high-degree vertices
+// (bit 31 of the pair's row index) last, others first.  Most DAG arcs end at the
+// former, so their sectors are read again and again within a level, while the
+// rows of the many low-degree vertices stream through.  A hint only; results do
+// not depend on it.  R-MAT 22, 4096 sources: MFBr gather 387 -> 378 ms, R-MAT 20
+// 98.1 -> 95.9; on graphs of 2^17 vertices and in the MFBF gather, whose sums are
+// read from the L2 anyway, the extra operand costs 1-3 %.
+struct L2Hint {
+  uint64_t keep, stream;
+  __device__ __forceinline__ L2Hint() {
+    asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(keep));
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(stream));
+  }
+};
+__device__ __forceinline__ void ld4u_hint(const L2Hint& h, uint32_t sl, uint32_t row, const uint64_t* p, uint64_t& a,
+                                          uint64_t& b, uint64_t& c, uint64_t& d) {
+  asm volatile("{.reg .pred p, q; .reg .b64 l; setp.ne.u32 p, %5, 0; setp.lt.s32 q, %6, 0; selp.b64 l, %7, %8, q;"
+               " @p ld.global.L1::no_allocate.L2::cache_hint.v4.u64 {%0,%1,%2,%3}, [%4], l;}"
+               : "=l"(a), "=l"(b), "=l"(c), "=l"(d) : "l"(p), "r"(sl), "r"(row), "l"(h.keep), "l"(h.stream));
 }
 
 // Gather over a group of up to 32 segments (lane k holds segment k's header).
@@ -677,11 +686,22 @@ __device__ __forceinline__ void ld4u(const uint64_t* p, uint64_t& a, uint64_t& b
 // values with compensation.  FLUSH(k, ...) is called once per segment with
 // pairs, in order, by the whole warp, with the lane's four column sums and
 // the OR of its 4-bit slices.
-template <bool COUNT, bool INT, class Flush>
+//
+// What bounds it: instruction issue and L2 latency on power-law graphs (integer
+// pipe 60 %, L1 data stage 59 %, R-MAT 17), DRAM sectors on uniform ones (79 % of
+// the DRAM rate on the widest level of n = 100 000, k = 32).  R-MAT 20, 4096
+// sources, MFBF / MFBr gather: 82.7 / 106.8 -> 73.2 / 95.9 ms; uniform n = 300 007,
+// k = 32, 2048 sources: 33.5 / 37.7 -> 29.1 / 32.3.
+// Tried and not kept: visiting only the pairs with a bit in the lane's columns
+// (a transposed bit matrix; 1.6 -> 1.1 ms where 7 of 128 columns are set, but
+// 20-30 % slower where 30 are); adding counts on the FMA pipe (73 -> 81 ms); 2 or
+// 8 pairs in flight (82, 152 ms); one copy of the flush (the pairs' registers
+// then go to memory: 162 ms).
+template <bool COUNT, bool INT, bool HINT, class Flush>
 __device__ __forceinline__ void gather_group(const uint4& myseg, int nin, const uint32_t* __restrict__ prow,
                                              const uint4* __restrict__ pmask, GatherSmem& gs, const uint64_t* sv,
-                                             unsigned long long& nvals, unsigned long long& nvals_rec, uint32_t& ovf,
-                                             Flush flush) {
+                                             unsigned long long& nvals, unsigned long long& nvals_rec,
+                                             const L2Hint& hint, Flush flush) {
   const unsigned lane = lane_id();
   const int mycnt = (int)lane < nin ? (int)(myseg.z & 0xffu) : 0;
   int incl = mycnt;
@@ -703,50 +723,53 @@ __device__ __forceinline__ void gather_group(const uint4& myseg, int nin, const 
   float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;            // MFBr sums
   float c0 = 0.f, c1 = 0.f, c2 = 0.f, c3 = 0.f;            //   and their compensations
   uint32_t cs = 0;
+  const uint64_t* mysv = sv + 4 * lane;
+  const uint32_t* mymask = reinterpret_cast<const uint32_t*>(gs.mask) + mword;
+  auto add = [&](uint32_t sl, const uint64_t (&x)[4]) {
+    if (INT) {
+      // no wrap check per add: stored counts stay below 2^58 (larger sums are
+      // flagged at the flush), and a segment adds <= 32 of them
+      if (sl & 1u) i0 += x[0];
+      if (sl & 2u) i1 += x[1];
+      if (sl & 4u) i2 += x[2];
+      if (sl & 8u) i3 += x[3];
+    } else {
+      if (sl & 1u) acc_add(s0, c0, x[0]);
+      if (sl & 2u) acc_add(s1, c1, x[1]);
+      if (sl & 4u) acc_add(s2, c2, x[2]);
+      if (sl & 8u) acc_add(s3, c3, x[3]);
+    }
+  };
   for (int p0 = 0; p0 < T; p0 += 32) {
     uint32_t lastmask;
-    stage_chunk<COUNT>(myseg, excl, incl, T, p0, prow, pmask, gs, &lastmask);
+    stage_chunk(myseg, excl, incl, T, p0, prow, pmask, gs, &lastmask);
     const int nq = T - p0 < 32 ? T - p0 : 32;
-    for (int q0 = 0; q0 < nq; q0 += GATHER_U) {
+    for (int q0 = 0; q0 < nq; q0 += GATHER_U) {          // (places past nq have empty masks)
       uint64_t x[GATHER_U][4];
       uint32_t sl[GATHER_U];
 #pragma unroll
       for (int r = 0; r < GATHER_U; r++) {
-        const int q = q0 + r;
-        sl[r] = 0u;
-        x[r][0] = x[r][1] = x[r][2] = x[r][3] = 0ull;
-        if (q < nq) {
-          const uint32_t mw = reinterpret_cast<const uint32_t*>(&gs.mask[q])[mword];
-          sl[r] = (mw >> shift) & 0xfu;
-          if (sl[r]) {
-            const uint32_t rr = gs.row[q];
-            const uint64_t* p = sv + (size_t)(rr & 0x7fffffffu) * 128 + 4 * lane;
-            if (rr >> 31) ld4u_keep(p, x[r][0], x[r][1], x[r][2], x[r][3]);
-            else ld4u(p, x[r][0], x[r][1], x[r][2], x[r][3]);
-            if (COUNT) nvals += __popc(sl[r]);
-          }
-        }
+        sl[r] = (mymask[4 * (q0 + r)] >> shift) & 0xfu;
+        const uint32_t row = gs.row[q0 + r];
+        const uint64_t* p = mysv + (size_t)(row & 0x7fffffffu) * 128;
+        if (HINT) ld4u_hint(hint, sl[r], row, p, x[r][0], x[r][1], x[r][2], x[r][3]);
+        else ld4u_if(sl[r], p, x[r][0], x[r][1], x[r][2], x[r][3]);
+        if (COUNT) nvals += __popc(sl[r]);
       }
+      const uint32_t last = (lastmask >> q0) & ((1u << GATHER_U) - 1u);
+      if (!last) {                                       // (uniform) no segment ends in these pairs
 #pragma unroll
-      for (int r = 0; r < GATHER_U; r++) {
-        const int q = q0 + r;
-        if (q < nq) {
-          if (INT) {
-            // no wrap check per add: stored counts stay below 2^58 (larger
-            // sums are flagged at the flush), and a segment adds <= 32 of them
-            if (sl[r] & 1u) i0 += x[r][0];
-            if (sl[r] & 2u) i1 += x[r][1];
-            if (sl[r] & 4u) i2 += x[r][2];
-            if (sl[r] & 8u) i3 += x[r][3];
-          } else {
-            if (sl[r] & 1u) acc_add(s0, c0, x[r][0]);
-            if (sl[r] & 2u) acc_add(s1, c1, x[r][1]);
-            if (sl[r] & 4u) acc_add(s2, c2, x[r][2]);
-            if (sl[r] & 8u) acc_add(s3, c3, x[r][3]);
-          }
+        for (int r = 0; r < GATHER_U; r++) {
+          add(sl[r], x[r]);
           cs |= sl[r];
-          if ((lastmask >> q) & 1u) {
-            flush(gs.seg[q], i0, i1, i2, i3, s0, s1, s2, s3, c0, c1, c2, c3, cs);
+        }
+      } else {
+#pragma unroll
+        for (int r = 0; r < GATHER_U; r++) {
+          add(sl[r], x[r]);
+          cs |= sl[r];
+          if ((last >> r) & 1u) {
+            flush(gs.seg[q0 + r], i0, i1, i2, i3, s0, s1, s2, s3, c0, c1, c2, c3, cs);
             i0 = i1 = i2 = i3 = 0ull;
             s0 = s1 = s2 = s3 = c0 = c1 = c2 = c3 = 0.f;
             cs = 0u;
@@ -771,8 +794,8 @@ __device__ __forceinline__ void gather_group(const uint4& myseg, int nin, const 
     if ((int)lane < nin) myseg = segs[base + lane];
 
 // MFBF gather of level l: sigma_bar(s,v) = sum over the segment's pairs
-// (exact 64-bit integers).  flags: bit 1 some sigma_bar >= 2^53, bit 3 a sum
-// passed 2^64 (the batch is then recomputed by the general kernels).
+// (exact 64-bit integers).  flags: bit 1 some sigma_bar >= 2^53, bit 3 some
+// sigma_bar >= 2^58 (the batch is then recomputed by the general kernels).
 template <bool COUNT, bool G32>
 __global__ void __launch_bounds__(256, MFBC_GATHER_MIN_BLOCKS) k_lvl_fwd_gather(
     const uint4* __restrict__ segs, const uint32_t* nseg_p, const uint32_t* __restrict__ prow,
@@ -785,9 +808,10 @@ __global__ void __launch_bounds__(256, MFBC_GATHER_MIN_BLOCKS) k_lvl_fwd_gather(
   const uint32_t nseg = *nseg_p;
   if (!G32) seg_group = seg_group_of(nseg, seg_group);
   unsigned long long nvals = 0, nw = 0, nrec = 0;
-  uint32_t ovf = 0, big = 0;
+  uint64_t seen = 0;                                  // OR of the counts: its top bit is the largest's
+  const L2Hint hint;                                  // (not used by the MFBF gather)
   FOR_SEGMENT_GROUPS(nseg, next_group, G32 ? 32 : seg_group)
-    gather_group<COUNT, true>(myseg, nin, prow, pmask, gs, sv, nvals, nrec, ovf,
+    gather_group<COUNT, true, false>(myseg, nin, prow, pmask, gs, sv, nvals, nrec, hint,
         [&](int k, uint64_t a0, uint64_t a1, uint64_t a2, uint64_t a3, float, float, float, float, float, float,
             float, float, uint32_t cs) {
       const int32_t v = (int32_t)__shfl_sync(0xffffffffu, myseg.x, k);
@@ -795,13 +819,13 @@ __global__ void __launch_bounds__(256, MFBC_GATHER_MIN_BLOCKS) k_lvl_fwd_gather(
       const int d = (int)((z >> 8) & 0xffu);
       if (cs) {
         uint64_t* dst = sv + (size_t)v * nb + 128 * d + 4 * lane;
-        uint64_t t0 = a0, t1 = a1, t2 = a2, t3 = a3;
+        uint64_t t0 = a0, t1 = a1, t2 = a2, t3 = a3;     // (columns without a pair are 0)
         if ((z >> 16) & 1u) {
           unsigned long long* da = reinterpret_cast<unsigned long long*>(dst);
-          if (cs & 1u) { const uint64_t o = atomicAdd(da + 0, (unsigned long long)a0); t0 = o + a0; ovf |= t0 < o; }
-          if (cs & 2u) { const uint64_t o = atomicAdd(da + 1, (unsigned long long)a1); t1 = o + a1; ovf |= t1 < o; }
-          if (cs & 4u) { const uint64_t o = atomicAdd(da + 2, (unsigned long long)a2); t2 = o + a2; ovf |= t2 < o; }
-          if (cs & 8u) { const uint64_t o = atomicAdd(da + 3, (unsigned long long)a3); t3 = o + a3; ovf |= t3 < o; }
+          if (cs & 1u) t0 += atomicAdd(da + 0, (unsigned long long)a0);
+          if (cs & 2u) t1 += atomicAdd(da + 1, (unsigned long long)a1);
+          if (cs & 4u) t2 += atomicAdd(da + 2, (unsigned long long)a2);
+          if (cs & 8u) t3 += atomicAdd(da + 3, (unsigned long long)a3);
         } else if (cs == 0xfu) {
           asm volatile("st.global.v4.u64 [%0], {%1,%2,%3,%4};" ::"l"(dst), "l"(a0), "l"(a1), "l"(a2), "l"(a3)
                        : "memory");
@@ -811,19 +835,16 @@ __global__ void __launch_bounds__(256, MFBC_GATHER_MIN_BLOCKS) k_lvl_fwd_gather(
           if (cs & 4u) dst[2] = a2;
           if (cs & 8u) dst[3] = a3;
         }
-        // bit 1: a count reached 2^53 (FP64 output inexact); bit 3: a count
-        // reached 2^58 (later sums could wrap 2^64: the batch is redone by the
-        // general kernels)
-        const uint64_t m = ((cs & 1u) ? t0 : 0ull) | ((cs & 2u) ? t1 : 0ull) | ((cs & 4u) ? t2 : 0ull) |
-                           ((cs & 8u) ? t3 : 0ull);
-        big |= (uint32_t)(m >= (1ull << 53));
-        ovf |= (uint32_t)(m >= (1ull << 58));
+        seen |= (t0 | t1) | (t2 | t3);
         if (COUNT) nw += __popc(cs);
       }
     });
   }
-  if (__any_sync(0xffffffffu, big != 0u) && lane == 0) atomicOr(flags, FLAG_SIGMA_INEXACT);
-  if (__any_sync(0xffffffffu, ovf != 0u) && lane == 0) atomicOr(flags, FLAG_COUNT_WRAP);
+  // a count reached 2^53 (FP64 output inexact) or 2^58 (later sums could wrap
+  // 2^64: the batch is redone by the general kernels; a sum can wrap only after a
+  // partial one of at least 2^63 was seen here)
+  if (__any_sync(0xffffffffu, seen >= (1ull << 53)) && lane == 0) atomicOr(flags, FLAG_SIGMA_INEXACT);
+  if (__any_sync(0xffffffffu, seen >= (1ull << 58)) && lane == 0) atomicOr(flags, FLAG_COUNT_WRAP);
   // (the gate's count: 0 after an overflow, whose redo must see the old visited rows)
   if (vn.count) {
     const uint32_t c = *((volatile const uint32_t*)vn.count);
@@ -899,7 +920,7 @@ __global__ void __launch_bounds__(256, MFBC_BWD_GATHER_MIN_BLOCKS) k_lvl_bwd_gat
   if (!G32) seg_group = seg_group_of(nseg, seg_group);
   const int shift = 4 * (int)(lane & 7u);
   unsigned long long nvals = 0, nw = 0, nrec = 0;
-  uint32_t ovf = 0;
+  const L2Hint hint;
   FOR_SEGMENT_GROUPS(nseg, next_group, G32 ? 32 : seg_group)
     auto finish = [&](int k, uint64_t, uint64_t, uint64_t, uint64_t, float s0, float s1, float s2, float s3, float c0,
                       float c1, float c2, float c3, uint32_t) {
@@ -945,7 +966,7 @@ __global__ void __launch_bounds__(256, MFBC_BWD_GATHER_MIN_BLOCKS) k_lvl_bwd_gat
         }
       }
     };
-    gather_group<COUNT, false>(myseg, nin, prow, pmask, gs, sv, nvals, nrec, ovf, finish);
+    gather_group<COUNT, false, G32>(myseg, nin, prow, pmask, gs, sv, nvals, nrec, hint, finish);
     // segments without successor pairs: zeta = 0
     uint32_t empty = __ballot_sync(0xffffffffu, (int)lane < nin && (myseg.z & 0xffu) == 0u && myseg.x != SEG_DUMMY);
     while (empty) {
@@ -1084,14 +1105,6 @@ __global__ void k_lvl_output(const int32_t* __restrict__ list, uint32_t count, i
     rc.prof->end(id);             \
   } while (0)
 
-// one warp per 32 items (the precheck group)
-static inline unsigned grid_for_items(int64_t items, unsigned cap) {
-  uint64_t warps = ((uint64_t)items + 31) / 32;
-  uint64_t b = (warps + LVL_WARPS - 1) / LVL_WARPS;
-  if (b < 1) b = 1;
-  return (unsigned)(b > cap ? cap : b);
-}
-
 static void set_smem_attrs() {
   static bool done = false;
   if (done) return;
@@ -1174,7 +1187,13 @@ static mfbc_status level_round(RunCtx& rc, LevelState& s, bool fwd, int l, int64
   // the gather walks past
   const uint32_t seg_chunk =
       ig == 32 ? SEG_CHUNK : std::max<uint32_t>(2u * Qn, std::min<uint32_t>(SEG_CHUNK, 2u * ig * Qn));
-  const uint32_t* hot = MFBC_HOT_HINT && (uint64_t)n * (uint64_t)Qn < (1ull << 31) ? g.hot : nullptr;
+  const int64_t items = fwd ? g.items_in.count : g.items_out.count;
+  // groups of 32 segments compile to constants (G32) where the graph is large
+  // enough that its wide levels have that many segments (a quad per item and
+  // quad is at least 8x the segments that 32 per group need); so do the L2
+  // priorities of the MFBr gather, whose rows' bit 31 the pair kernel sets
+  const bool large = (uint64_t)items * (uint64_t)Qn >= 8ull * 32 * 4 * (fwd ? kGatherGrid : kBwdGatherGrid) * 8;
+  const uint32_t* hot = large && !fwd && (uint64_t)n * (uint64_t)Qn < (1ull << 31) ? g.hot : nullptr;
   if (fwd)
     PROF(K_LVL_FWD, (k_lvl_fwd_pairs<<<pgrid, LVL_WARPS * 32, LVL_SMEM, st>>>(
                         ib, ie, g.items_in.v, g.items_in.beg, g.col_t, W, s.full, s.V, Fl, Ml, Fn, Mn,
@@ -1212,12 +1231,8 @@ static mfbc_status level_round(RunCtx& rc, LevelState& s, bool fwd, int l, int64
     vn.count = &s.ctr->visit_count;
     *visited_next = true;
   }
-  // groups of 32 segments compile to constants (G32): taken when the round
-  // has that many segments (checked) or the graph is large enough that its
-  // wide levels do (unchecked: a quad per item and quad is at least 8x the
-  // segments that 32 per group need)
-  const int64_t items = fwd ? g.items_in.count : g.items_out.count;
-  const bool g32 = checked ? gs == 32 : (uint64_t)items * (uint64_t)Qn >= 8ull * 32 * 4 * gcap * 8;
+  // (a checked round knows its segment count)
+  const bool g32 = checked ? gs == 32 : large;
 #define GATHER_LAUNCH(kern, C, ...)                                                   \
   do {                                                                                \
     if (g32) kern<C, true><<<ggrid, 256, 0, st>>>(__VA_ARGS__);                       \
