@@ -1045,9 +1045,9 @@ mfbc_status run(mfbc_graph* G, const int32_t* d_src, int32_t nsrc, int mode, dou
 
 // The level gathers read scattered 32-byte sectors; with the context's
 // default L2 fetch granularity (64 bytes) a miss also brings in the
-// neighbouring sector, which is mostly not needed (measured: 5 % slower on
-// R-MAT 22).  A call sets the hint to 32 bytes while it runs and restores the
-// previous value when it returns (its work is complete by then).
+// neighbouring sector, which is mostly not needed.  A call sets the hint to 32
+// bytes while it runs and restores the previous value when it returns (its work
+// is complete by then).
 struct L2FetchHint {
   size_t prev = 0;
   bool set = false;
@@ -1062,6 +1062,22 @@ struct L2FetchHint {
     if (set && cudaDeviceSetLimit(cudaLimitMaxL2FetchGranularity, prev) != cudaSuccess) cudaGetLastError();
   }
 };
+
+// Which calls set the hint.  The two driver calls cost 0.73 ms together, and
+// the hint gives that back only where the gathers miss the L2 for long enough:
+// the {sigma} state of a batch (8 n n_b bytes) well above the 129 MB that the
+// L2 holds, and enough of it over all batches.  With hubs most gathers hit the
+// rows of a few vertices, which the L2 keeps, so the line lies higher.  Call
+// with the hint against without it, in ms: uniform graphs of average degree 16,
+// 100 000 vertices x 1024 columns (0.8 GB) 9.57 / 9.89, 300 000 vertices
+// 79 / 95; R-MAT, one batch each: 14 x 1024 (0.13 GB) 2.89 / 2.16, 17 (1.1 GB)
+// 13.5 / 12.8, 18 x 1024 (2.1 GB) 22.6 / 22.4; two batches of 19 (4.3 GB each) 61.5 / 61.9;
+// 20 220 / 228.
+static bool wants_l2_hint(const DevGraph& g, const Plan& p, int32_t nsrc) {
+  if (p.path != MFBC_PATH_LEVEL || p.by_source) return false;
+  const double row = 8.0 * (double)g.n, batch = row * p.nb, all = row * std::max(nsrc, p.nb);
+  return has_hubs(g) ? batch >= 2e9 && all >= 4e9 : batch >= 0.7e9;
+}
 
 mfbc_status entry(const mfbc_graph* Gc, const int32_t* sources, int32_t nsrc, int mode, double* lambda_out,
                   int32_t* dist_out, double* sigma_out, const mfbc_options* opt, bool host_io,
@@ -1108,10 +1124,8 @@ mfbc_status entry(const mfbc_graph* Gc, const int32_t* sources, int32_t nsrc, in
   if (s) return s;
   s = get_workspace(R);
   if (s) return s;
-  // only the level kernels' gathers gain from the 32-byte fetch hint; setting
-  // and restoring it costs two driver calls that small calls would feel
   std::optional<L2FetchHint> l2hint;
-  if (R.plan.path == MFBC_PATH_LEVEL && !R.plan.by_source) l2hint.emplace();
+  if (wants_l2_hint(G->g, R.plan, nsrc)) l2hint.emplace();
   R.prof.on = opt && opt->profile;
   R.prof.count_bytes = R.prof.on && (opt->flags & MFBC_OPT_COUNT_BYTES);
   R.prof.stream = R.st;
