@@ -132,6 +132,40 @@ def test_forms_match_oracle(name):
         G.close()
 
 
+def unit(g):
+    return gg.CSRGraph(n=g.n, rowptr=g.rowptr, col=g.col, w=None, directed=g.directed)
+
+
+# without weights: tau in 16-bit, 8-bit (a source deeper than 254 levels is redone
+# wide) and global memory; more DAG arcs than are recorded; rows the warps share
+UNIT_CASES = {
+    "smem16": lambda: (gg.erdos_renyi(40001, 12, seed=21), 20),
+    "smem16_directed": lambda: (gg.rmat(11, 8, directed=True, seed=22), 60),
+    "smem8": lambda: (gg.erdos_renyi(120001, 10, seed=23), 9),
+    "smem8_redone_wide": lambda: (unit(with_tail(gg.erdos_renyi(120001, 10, weights=(1, 2), seed=24), 300, 1)), 9),
+    "global": lambda: (gg.erdos_renyi(120001, 4, seed=25), 9),
+    "dag_overflows": lambda: (gg.erdos_renyi(300, 290, seed=26), 40),
+    "hub_list_overflows": lambda: (unit(hubs(100, 600, False, 27)), 30),
+    "hub_list_overflows_directed": lambda: (unit(hubs(100, 600, True, 28)), 30),
+}
+
+
+@pytest.mark.parametrize("name", UNIT_CASES)
+def test_unit_forms_match_oracle(name):
+    g, k = UNIT_CASES[name]()
+    srcs = np.concatenate([[0], gg.sample_sources(g, k, seed=3)]).astype(np.int32)
+    want = oracle.bc(g, srcs)
+    wd, ws, _ = oracle.sssp(g, srcs[:20])
+    G = mfbc.Graph.from_csr(g)
+    try:
+        for p in (mfbc.PATH_SMALL, mfbc.PATH_AUTO):
+            close(G.bc(srcs, path=p), want)
+            d, s = G.sssp(srcs[:20], path=p)
+            assert np.array_equal(d, wd) and np.array_equal(s, ws)
+    finally:
+        G.close()
+
+
 def test_workspaces_of_any_accepted_size():
     # a caller's workspace sized for many sources serves few, and one as small
     # as the narrowest width's serves all
