@@ -338,16 +338,19 @@ static bool general_by_source(const DevGraph& g, int32_t nsrc) {
 }
 
 // The level kernels share a frontier's bit rows and arcs among the columns of a
-// batch but pay 1.2 ms of launches for a batch however small; one block per
-// source pays every arc for every source.  Milliseconds level / source kernel
-// at 1, 64, 152, 304, 456 sources: R-MAT 14 (4.3 * 10^5 arcs) 1.4 / 0.5, 1.8 /
-// 0.7, 2.0 / 0.7, 2.2 / 1.2, 2.4 / 2.0; uniform n = 20 000, k = 60 1.3 / 1.1,
-// 1.8 / 1.2, 2.2 / 1.2, 2.6 / 2.3, 3.1 / 4.4; uniform n = 60 000, k = 8 2.0 /
-// 1.0, 2.6 / 1.0, 3.0 / 1.3, 3.7 / 3.0, 4.3 / 6.1; directed R-MAT 16 (9.6 * 10^5)
-// 1.7 / 1.3, 2.2 / 1.7, 2.6 / 1.8, 3.3 / 3.4; R-MAT 16 (1.8 * 10^6) 1.8 / 2.3,
-// 2.8 / 2.5; uniform n = 16 000, k = 10, 500 / 2000 sources 2.2 / 1.3, 5.8 / 4.7.
+// batch but pay 0.5 ms of launches for a batch however small and more for every
+// level; one block per source pays every arc for every source.  Milliseconds
+// level / source kernel at 1, 64, 152, 304, 456 sources: R-MAT 14 (4.3 * 10^5
+// arcs) 0.8 / 0.5, 1.1 / 0.7, 1.2 / 0.7, 1.4 / 1.3, 1.6 / 2.0; uniform n = 60 000,
+// k = 8 1.4 / 1.0, 1.8 / 1.0, 2.2 / 1.2, 2.8 / 2.7, 3.4 / 4.1; n = 16 000, k = 10,
+// 304 / 456 / 1000 sources 1.3 / 0.6, 1.5 / 1.0, 2.0 / 1.9.  With more arcs the
+// two are close up to 152 sources (n = 100 000, k = 8 1.4 / 1.5, 2.2 / 1.7, 2.9 /
+// 2.4) or the level kernels win (n = 20 000, k = 60 0.7 / 1.2, 1.1 / 1.3, 1.4 /
+// 1.3; R-MAT 15 0.9 / 0.9, 1.2 / 1.3, 1.6 / 1.4), unless the graph is sparse
+// enough to be deep (n = 600 000, k = 2 5.8 / 4.5, 14 / 5.4, 21 / 10).
 static bool level_by_source(const DevGraph& g, int32_t nsrc) {
-  return g.nnz <= 1250000 && (nsrc <= 152 || (int64_t)nsrc * g.nnz <= 130000000);
+  return g.nnz <= (g.nnz <= 3 * (int64_t)g.n ? 1250000 : 600000) &&
+         (nsrc <= 152 || (int64_t)nsrc * g.nnz <= 130000000);
 }
 
 static int tuned_slot(int path) {
