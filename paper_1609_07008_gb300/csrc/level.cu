@@ -221,10 +221,11 @@ __global__ void k_lvl_round_gate(uint32_t* work, const uint32_t* list_count, uin
 }
 
 // Per-warp shared memory of the pair kernels.
-struct WarpSmem {
+struct alignas(16) WarpSmem {
   int32_t su[32];                            // member neighbour ids of the item
   int32_t newv[32];                          // vertices entering the next level, not yet appended
-  uint32_t sF[32][33];                       // member q's masked frontier word j (padded: no bank conflicts)
+  uint32_t sF[32][36];                       // member q's masked frontier word j (padded: a quad of every
+                                             // row is read as 16 bytes a lane without bank conflicts)
 };
 constexpr size_t LVL_SMEM = sizeof(WarpSmem) * LVL_WARPS;
 
@@ -254,12 +255,36 @@ __device__ __forceinline__ bool meta_multi(int64_t m) { return (m >> 46) & 1; }
 // Pair record: row index (uint32) and the 128-column mask (uint4, word w of
 // the quad in component w).  Segment header: (v, first pair, count | quad << 8
 // | multi-item row << 16, 0); a segment is one (vertex, quad) of one work item.
-__device__ __forceinline__ uint4 make_seg(int32_t v, uint32_t pb, int cnt, int d, bool multi) {
-  return make_uint4((uint32_t)v, pb, (uint32_t)cnt | ((uint32_t)d << 8) | ((uint32_t)multi << 16), 0u);
-}
 
-__device__ __forceinline__ uint32_t quad_or(const WarpSmem& w, int q, int d) {
-  return w.sF[q][4 * d] | w.sF[q][4 * d + 1] | w.sF[q][4 * d + 2] | w.sF[q][4 * d + 3];
+// words 4d..4d+3 of member q's masked frontier row
+__device__ __forceinline__ uint4 quad_of(const WarpSmem& w, int q, int d) {
+  return *reinterpret_cast<const uint4*>(&w.sF[q][4 * d]);
+}
+__device__ __forceinline__ bool any_bit(const uint4& m) { return (m.x | m.y | m.z | m.w) != 0u; }
+
+// The rows F(u) & mask of the item's nm members (ids in sm.su) into sm.sF, eight
+// in flight; returns their OR (this lane's word).  Lanes past W read the last
+// word and have an empty mask; rows up to the next multiple of eight become zero.
+__device__ __forceinline__ uint32_t stage_rows(WarpSmem& sm, int nm, int W, const uint32_t* __restrict__ F,
+                                               uint32_t mask) {
+  const unsigned lane = lane_id();
+  const uint32_t* Fw = F + min((int)lane, W - 1);
+  uint32_t any = 0;
+  for (int q0 = 0; q0 < nm; q0 += 8) {
+    int32_t u[8];
+    *reinterpret_cast<int4*>(u) = *reinterpret_cast<const int4*>(&sm.su[q0]);
+    *reinterpret_cast<int4*>(u + 4) = *reinterpret_cast<const int4*>(&sm.su[q0 + 4]);
+    uint32_t f[8];
+#pragma unroll
+    for (int t = 0; t < 8; t++) f[t] = q0 + t < nm ? __ldg(Fw + (size_t)u[t] * W) : 0u;
+#pragma unroll
+    for (int t = 0; t < 8; t++) {
+      sm.sF[q0 + t][lane] = f[t] & mask;
+      any |= f[t] & mask;
+    }
+  }
+  __syncwarp();
+  return any;
 }
 
 // Pair and segment slots reserved by one warp.  Slots are taken from the
@@ -295,6 +320,13 @@ __device__ __forceinline__ void fill_dummy_segs(uint4* segs, uint32_t b, uint32_
 // Emit the (member, mask) pairs of one item, quad by quad over `quads`
 // (ascending), as segments.  Returns false (writing nothing) when the
 // buffers are full.
+//
+// The pair kernels are bound by instruction issue (2.8 of 4 a cycle, R-MAT 17):
+// a quad's words come as one 16-byte read a lane, the pairs are counted as they
+// are written, and ahead of that only where the warp's slots might not suffice
+// for all members in all quads.  MFBF / MFBr pair kernels, R-MAT 20, 4096 sources:
+// 20.8 / 15.2 -> 16.6 / 12.1 ms; directed R-MAT 17, 1536 sources: 1.49 / 1.22 ->
+// 1.24 / 1.00.
 __device__ __forceinline__ bool emit_quads(const WarpSmem& w, int nm, int32_t v, bool multi, uint32_t quads, int Q,
                                            const uint32_t* __restrict__ hot, uint32_t* prow, uint4* pmask,
                                            uint4* segs, uint32_t* work,
@@ -302,45 +334,49 @@ __device__ __forceinline__ bool emit_quads(const WarpSmem& w, int nm, int32_t v,
                                            unsigned long long* npairs, uint32_t seg_chunk) {
   const unsigned lane = lane_id();
   const uint32_t lt = (1u << lane) - 1u;
-  int mycnt = 0;
-  for (uint32_t ql = quads; ql; ql &= ql - 1) {
-    const int d = __ffs(ql) - 1;
-    const uint32_t mk = __ballot_sync(0xffffffffu, ((int)lane < nm) && quad_or(w, lane, d) != 0u);
-    if ((int)lane == d) mycnt = __popc(mk);
-  }
-  int incl = mycnt;
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, incl, o);
-    if ((int)lane >= o) incl += y;
-  }
-  const int excl = incl - mycnt;
-  const uint32_t P = (uint32_t)__shfl_sync(0xffffffffu, incl, 31);
+  const bool mine = (int)lane < nm;
   const uint32_t S = (uint32_t)__popc(quads);
-  if (cur.p + P > cur.pe && !reserve_slots(&work[0], P, PAIR_CHUNK, pair_cap, &work[3], cur.p, cur.pe))
-    return false;
+  if (cur.p + (uint32_t)nm * S > cur.pe) {
+    uint32_t P = 0;
+    for (uint32_t ql = quads; ql; ql &= ql - 1)
+      P += __popc(__ballot_sync(0xffffffffu, mine && any_bit(quad_of(w, lane, __ffs(ql) - 1))));
+    if (cur.p + P > cur.pe && !reserve_slots(&work[0], P, PAIR_CHUNK, pair_cap, &work[3], cur.p, cur.pe))
+      return false;
+  }
   if (cur.s + S > cur.se) {
     fill_dummy_segs(segs, cur.s, cur.se);
     if (!reserve_slots(&work[1], S, seg_chunk, seg_cap, &work[3], cur.s, cur.se)) return false;
   }
-  const uint32_t pb = cur.p, sb = cur.s;
-  cur.p += P;
-  cur.s += S;
-  // bit 31 of a pair's row index: the row belongs to a high-degree vertex
-  const uint32_t hotbit = ((int)lane < nm && hot && test_bit(hot, w.su[lane])) ? 0x80000000u : 0u;
-  if (npairs) *npairs += P + (uint64_t)S * (1ull << 32);   // pairs in the low word, segments in the high
+  const uint32_t pb = cur.p;
+  uint32_t row = 0;                              // of this lane's member, quad 0
+  if (mine) {
+    // bit 31 of a pair's row index: the row belongs to a high-degree vertex
+    row = (uint32_t)w.su[lane] * (uint32_t)Q;
+    if (hot && test_bit(hot, w.su[lane])) row |= 0x80000000u;
+  }
+  uint32_t sp = 0, sz = 0;                       // lane r: segment r's first pair, its pairs and quad
   int r = 0;
   for (uint32_t ql = quads; ql; ql &= ql - 1, r++) {
     const int d = __ffs(ql) - 1;
-    const bool nz = ((int)lane < nm) && quad_or(w, lane, d) != 0u;
+    uint4 m = make_uint4(0u, 0u, 0u, 0u);
+    if (mine) m = quad_of(w, lane, d);
+    const bool nz = any_bit(m);
     const uint32_t mk = __ballot_sync(0xffffffffu, nz);
-    const uint32_t off = (uint32_t)__shfl_sync(0xffffffffu, excl, d);
     if (nz) {
-      const uint32_t at = pb + off + __popc(mk & lt);
-      prow[at] = ((uint32_t)w.su[lane] * (uint32_t)Q + (uint32_t)d) | hotbit;
-      pmask[at] = make_uint4(w.sF[lane][4 * d], w.sF[lane][4 * d + 1], w.sF[lane][4 * d + 2], w.sF[lane][4 * d + 3]);
+      const uint32_t at = cur.p + __popc(mk & lt);
+      prow[at] = row + (uint32_t)d;
+      pmask[at] = m;
     }
-    if (lane == 0) segs[sb + r] = make_seg(v, pb + off, __popc(mk), d, multi);
+    const uint32_t cnt = (uint32_t)__popc(mk);
+    if ((int)lane == r) {
+      sp = cur.p;
+      sz = cnt | ((uint32_t)d << 8);
+    }
+    cur.p += cnt;
   }
+  if (lane < S) segs[cur.s + lane] = make_uint4((uint32_t)v, sp, sz | ((uint32_t)multi << 16), 0u);
+  cur.s += S;
+  if (npairs) *npairs += (cur.p - pb) + (uint64_t)S * (1ull << 32);   // pairs in the low word, segments in the high
   return true;
 }
 
@@ -445,22 +481,7 @@ __global__ void __launch_bounds__(LVL_WARPS * 32, MFBC_PAIR_MIN_BLOCKS) k_lvl_fw
       const int nm = __popc(mm);
       if (isMem) sm.su[__popc(mm & lt)] = u;
       __syncwarp();
-      uint32_t cand = 0;
-      for (int q0 = 0; q0 < nm; q0 += 8) {          // eight frontier rows in flight
-        uint32_t f[8];
-#pragma unroll
-        for (int t = 0; t < 8; t++)
-          f[t] = (q0 + t < nm && (int)lane < W) ? __ldg(&Fl[(size_t)sm.su[q0 + t] * W + lane]) : 0u;
-#pragma unroll
-        for (int t = 0; t < 8; t++) {
-          if (q0 + t < nm) {
-            const uint32_t mk = f[t] & ~Vv;
-            sm.sF[q0 + t][lane] = mk;
-            cand |= mk;
-          }
-        }
-      }
-      __syncwarp();
+      const uint32_t cand = stage_rows(sm, nm, W, Fl, ~Vv);
       if (bytes) nbytes += 4ull * W * (nm + 1);
       const uint32_t cw = __ballot_sync(0xffffffffu, cand != 0u);
       if (!cw) continue;
@@ -556,21 +577,7 @@ __global__ void __launch_bounds__(LVL_WARPS * 32, MFBC_PAIR_MIN_BLOCKS) k_lvl_bw
       const int nm = __popc(mm);
       if (isMem) sm.su[__popc(mm & lt)] = u;
       __syncwarp();
-      uint32_t any = 0;
-      for (int q0 = 0; q0 < nm; q0 += 8) {          // eight frontier rows in flight
-        uint32_t f[8];
-#pragma unroll
-        for (int t = 0; t < 8; t++)
-          f[t] = (q0 + t < nm && (int)lane < W) ? __ldg(&Fn[(size_t)sm.su[q0 + t] * W + lane]) : 0u;
-#pragma unroll
-        for (int t = 0; t < 8; t++) {
-          if (q0 + t < nm) {
-            sm.sF[q0 + t][lane] = f[t] & Fv;
-            any |= f[t] & Fv;
-          }
-        }
-      }
-      __syncwarp();
+      const uint32_t any = stage_rows(sm, nm, W, Fn, Fv);
       if (bytes) nbytes += 4ull * W * (nm + 1);
       const uint32_t words = __ballot_sync(0xffffffffu, multi ? any != 0u : Fv != 0u);
       if (words) emit_quads(sm, nm, v, multi, quads_of_words(words, Q), Q, hot, prow, pmask, segs, work, pair_cap,
