@@ -16,6 +16,7 @@ struct mfbc_graph {
   void* ws = nullptr;              // cached scratch (cudaMalloc), grown on demand
   size_t ws_bytes = 0;
   uint32_t* h_ctr = nullptr;       // pinned counter mirror
+  cudaEvent_t ev[2] = {nullptr, nullptr};   // reads of two level rounds in flight
   uint32_t flags = 0;
   std::mutex mu;
   // autotuner results (mfbc_autotune): batch width per kernel family
@@ -85,6 +86,12 @@ static mfbc_status csc_to_csr(int32_t n, int64_t nnz, const int64_t* rp, const i
   return MFBC_OK;
 }
 
+static void free_mirror(mfbc_graph* G) {
+  if (G->h_ctr) cudaFreeHost(G->h_ctr);
+  for (cudaEvent_t ev : G->ev)
+    if (ev) cudaEventDestroy(ev);
+}
+
 static mfbc_status create_common(int32_t n, int64_t nnz, const int64_t* rowptr, const int32_t* col,
                                  const int32_t* w, uint32_t flags, void* stream, mfbc_graph** out) {
   std::vector<int64_t> trp;
@@ -101,12 +108,14 @@ static mfbc_status create_common(int32_t n, int64_t nnz, const int64_t* rowptr, 
   std::string err;
   mfbc_status s = graph_build(n, nnz, rowptr, col, w, flags, (cudaStream_t)stream, &G->g, &err);
   if (s == MFBC_OK) {
-    cudaError_t e = cudaMallocHost((void**)&G->h_ctr, 64);
-    if (e != cudaSuccess) { s = MFBC_ERR_OOM; err = "cudaMallocHost of the counter mirror failed"; }
+    cudaError_t e = cudaMallocHost((void**)&G->h_ctr, 2 * ROUND_WORDS * sizeof(uint32_t));
+    for (cudaEvent_t& ev : G->ev)
+      if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+    if (e != cudaSuccess) { s = MFBC_ERR_OOM; err = "allocation of the counter mirror failed"; }
   }
   if (s != MFBC_OK) {
     graph_free(&G->g);
-    if (G->h_ctr) cudaFreeHost(G->h_ctr);
+    free_mirror(G);
     delete G;
     cudaGetLastError();
     return fail(s, err);
@@ -161,7 +170,7 @@ extern "C" void mfbc_graph_destroy(mfbc_graph* G) {
   if (!G) return;
   graph_free(&G->g);
   if (G->ws) cudaFree(G->ws);
-  if (G->h_ctr) cudaFreeHost(G->h_ctr);
+  free_mirror(G);
   delete G;
 }
 
@@ -853,7 +862,7 @@ mfbc_status run(mfbc_graph* G, const int32_t* d_src, int32_t nsrc, int mode, dou
   const Plan& P = R.plan;
   const int nb = P.nb;
   int64_t batches = 0, fi = 0, bi = 0;
-  RunCtx rc{&g, R.st, &R.prof, G->h_ctr, &R.err};
+  RunCtx rc{&g, R.st, &R.prof, G->h_ctr, &R.err, G->ev};
   rc.arcs = G->force_arcs ? G->force_arcs : G->tuned_arcs;
   rc.accum = R.opt && R.opt->accumulator ? R.opt->accumulator : G->tuned_accum;
   rc.small_rounds = R.opt && (R.opt->flags & MFBC_OPT_TEST_SMALL_ROUNDS);

@@ -82,6 +82,7 @@ constexpr uint32_t FLAG_COUNT_WRAP = 8u;     // level kernels: a path count reac
 constexpr uint32_t FLAG_TIMEOUT = 16u;       // a bounded device-side wait ran out (MFBC_ERR_TIMEOUT)
 constexpr uint32_t FLAG_ROUND_ABORT = 32u;   // level kernels: a round's pair buffers overflowed; the
                                              // launches queued after it return at once until cleared
+constexpr uint32_t FLAG_FWD_DONE = 64u;      // level kernels: the MFBF sweep has ended; rounds queued behind do nothing
 
 // Device-side counters of algorithmic bytes, one slot per kernel id.
 struct Counters {
@@ -90,9 +91,15 @@ struct Counters {
   uint32_t list_count[4];          // frontier / touched list sizes
   uint32_t flags;                  // FLAG_* bits
   uint32_t work[4];                // level kernels: pairs, segments, gather group counter, overflow
-  uint32_t abort_level;            // level kernels: highest MFBr level whose round overflowed
-  uint32_t visit_count;            // level kernels: vertices of the next level's visit (0 after an overflow)
+  // level kernels (what the host reads of a round are the 16 words from list_count):
+  uint32_t abort_level;            // highest MFBr level whose round overflowed
+  uint32_t visit_count;            // vertices of the next level's visit (0 after an overflow)
+  uint32_t gather_segs;            // segments of the round's gather
+  uint32_t round[2][2];            // MFBF round of level l at l & 1: the next level's size, overflow
+  unsigned long long fwd_off;      // where the next MFBF round's level list begins
+  unsigned long long visit_off;    //   and that of the running round's
 };
+constexpr int ROUND_WORDS = 16;
 
 class Profiler {
  public:
@@ -273,8 +280,10 @@ struct RunCtx {
   const DevGraph* g;
   cudaStream_t stream;
   Profiler* prof;
-  uint32_t* h_ctr;                 // pinned host mirror of Counters::list_count / flags
+  uint32_t* h_ctr;                 // pinned host mirror of Counters::list_count / flags (2 x ROUND_WORDS)
   std::string* err;
+  // level kernels: reads of two rounds in flight (null: every read waits for the stream)
+  const cudaEvent_t* ev = nullptr;
   // Requests packed into the current batch (host array, one entry per
   // 32-column word: the request owning the word's columns, -1 for none).
   // Request r adds into lambda + r * n.  nullptr: the whole batch is
