@@ -65,9 +65,16 @@ __device__ __forceinline__ uint64_t df_pack(dfl a) {
 __device__ __forceinline__ dfl df_unpack(uint64_t u) {
   return {__uint_as_float((uint32_t)u), __uint_as_float((uint32_t)(u >> 32))};
 }
-__device__ __forceinline__ dfl df_of_double(double x) {
-  const float h = __double2float_rn(x);
-  return {h, __double2float_rn(x - (double)h)};
+// x = 0 or 2^-74 <= x < 2^127 as hi + lo, hi = x rounded to FP32, lo = the
+// remainder rounded to FP32, on the integer pipe: hi takes the upper 23 mantissa
+// bits, rounded, lo the 29 below them as a signed number.  (FP64 conversions and
+// subtractions run at two a clock and SM.)
+__device__ __forceinline__ dfl df_of_positive(double x) {
+  const uint64_t u = (uint64_t)__double_as_longlong(x);
+  const uint32_t hi = (uint32_t)((u + (1ull << 28)) >> 29) - ((1023u - 127u) << 23);
+  const int rest = (int)((uint32_t)u << 3) >> 3;
+  const uint32_t scale = ((uint32_t)(u >> 52) - (1023u + 52u - 127u)) << 23;        // 2^(exponent - 52)
+  return u ? dfl{__uint_as_float(hi), __int2float_rn(rest) * __uint_as_float(scale)} : dfl{0.f, 0.f};
 }
 // compensated accumulation of non-negative double-float terms (hi, lo) into
 // (s, c): Fast2Sum on the ordered pair (max, min) gives the exact rounding
