@@ -297,25 +297,66 @@ __device__ __forceinline__ uint4 quad_of(const WarpSmem& w, int q, int d) {
 }
 __device__ __forceinline__ bool any_bit(const uint4& m) { return (m.x | m.y | m.z | m.w) != 0u; }
 
-// The rows F(u) & mask of the item's nm members (ids in sm.su) into sm.sF, eight
-// in flight; returns their OR (this lane's word).  Lanes past W read the last
-// word and have an empty mask; rows up to the next multiple of eight become zero.
-__device__ __forceinline__ uint32_t stage_rows(WarpSmem& sm, int nm, int W, const uint32_t* __restrict__ F,
-                                               uint32_t mask) {
+// A lane's place in the rows of narrow batches: word `word` of row `row` of the
+// `rows` (a power of two) that a warp reads at once.
+struct RowLanes {
+  int rows, row, word;
+  __device__ __forceinline__ explicit RowLanes(int W) {
+    rows = W <= 4 ? 8 : 4;
+    row = (int)lane_id() / W;
+    word = (int)lane_id() - row * W;
+  }
+};
+
+// The rows F(u) & mask of the item's nm members (ids in sm.su) into sm.sF;
+// returns their OR (this lane's word; 0 past W).
+// A warp reads one row eight times before it needs the first, or, with up to
+// NARROW_W words (256 columns), several rows at once, four times.  MFBF / MFBr
+// pair kernels of a call, one row against several: R-MAT 18, 100 sources 0.77 /
+// 0.61 -> 0.67 / 0.50 ms, 256 sources 0.85 / 0.70 -> 0.77 / 0.61, 384 (two rows) 0.96 /
+// 0.79 -> 0.95 / 0.80; R-MAT 20, 128 sources 3.00 / 2.48 -> 2.49 / 1.91.  (A kernel of
+// its own: as a branch, the wide form lost 5-20 %.)
+constexpr int NARROW_W = 8;
+template <bool NARROW>
+__device__ __forceinline__ uint32_t stage_rows(WarpSmem& sm, int nm, int W, const RowLanes& rl,
+                                               const uint32_t* __restrict__ F, uint32_t mask) {
   const unsigned lane = lane_id();
-  const uint32_t* Fw = F + min((int)lane, W - 1);
   uint32_t any = 0;
-  for (int q0 = 0; q0 < nm; q0 += 8) {
-    int32_t u[8];
-    *reinterpret_cast<int4*>(u) = *reinterpret_cast<const int4*>(&sm.su[q0]);
-    *reinterpret_cast<int4*>(u + 4) = *reinterpret_cast<const int4*>(&sm.su[q0 + 4]);
-    uint32_t f[8];
+  if (NARROW) {
+    const uint32_t m = __shfl_sync(0xffffffffu, mask, rl.word);
+    const uint32_t* Fw = F + rl.word;
+    const int own = rl.row < rl.rows ? nm : 0;       // (lanes past the last whole row are idle)
+    for (int q0 = 0; q0 < nm; q0 += 4 * rl.rows) {
+      uint32_t f[4];
 #pragma unroll
-    for (int t = 0; t < 8; t++) f[t] = q0 + t < nm ? __ldg(Fw + (size_t)u[t] * W) : 0u;
+      for (int t = 0; t < 4; t++) {
+        const int q = q0 + t * rl.rows + rl.row;
+        f[t] = q < own ? __ldg(Fw + (size_t)sm.su[q] * W) : 0u;
+      }
 #pragma unroll
-    for (int t = 0; t < 8; t++) {
-      sm.sF[q0 + t][lane] = f[t] & mask;
-      any |= f[t] & mask;
+      for (int t = 0; t < 4; t++) {
+        const int q = q0 + t * rl.rows + rl.row;
+        if (q < own) sm.sF[q][rl.word] = f[t] & m;
+        any |= f[t] & m;
+      }
+    }
+    for (int o = rl.rows / 2 * W; o >= W; o >>= 1) any |= __shfl_down_sync(0xffffffffu, any, o);
+    if ((int)lane >= W) any = 0u;
+  } else {
+    // (lanes past W read the last word and have an empty mask)
+    const uint32_t* Fw = F + min((int)lane, W - 1);
+    for (int q0 = 0; q0 < nm; q0 += 8) {
+      int32_t u[8];
+      *reinterpret_cast<int4*>(u) = *reinterpret_cast<const int4*>(&sm.su[q0]);
+      *reinterpret_cast<int4*>(u + 4) = *reinterpret_cast<const int4*>(&sm.su[q0 + 4]);
+      uint32_t f[8];
+#pragma unroll
+      for (int t = 0; t < 8; t++) f[t] = q0 + t < nm ? __ldg(Fw + (size_t)u[t] * W) : 0u;
+#pragma unroll
+      for (int t = 0; t < 8; t++) {
+        sm.sF[q0 + t][lane] = f[t] & mask;
+        any |= f[t] & mask;
+      }
     }
   }
   __syncwarp();
@@ -439,6 +480,7 @@ __device__ __forceinline__ uint32_t quads_of_words(uint32_t words, int Q) {
 // MFBF pairs of level l (see file comment): for items [ib, ie) of rows not yet
 // reached by every column, the masks F_l(u) & ~visited(v) of the in-neighbours
 // u in F_l, the next frontier bits F_{l+1}(v), and the level-(l+1) list.
+template <bool NARROW>
 __global__ void __launch_bounds__(LVL_WARPS * 32, MFBC_PAIR_MIN_BLOCKS) k_lvl_fwd_pairs(
     int64_t ib, int64_t ie, const int32_t* __restrict__ item_v, const int64_t* __restrict__ item_meta,
     const int32_t* __restrict__ col_t, int W, const uint32_t* __restrict__ full, const uint32_t* __restrict__ V,
@@ -452,6 +494,7 @@ __global__ void __launch_bounds__(LVL_WARPS * 32, MFBC_PAIR_MIN_BLOCKS) k_lvl_fw
   const unsigned lane = lane_id();
   const uint32_t lt = (1u << lane) - 1u;
   const int Q = W / 4;
+  const RowLanes rl(W);
   unsigned long long nbytes = 0, npairs = 0;
   SlotCursor cur;
   int nnew = 0;                                    // entries of sm.newv
@@ -519,7 +562,7 @@ __global__ void __launch_bounds__(LVL_WARPS * 32, MFBC_PAIR_MIN_BLOCKS) k_lvl_fw
       const int nm = __popc(mm);
       if (isMem) sm.su[__popc(mm & lt)] = u;
       __syncwarp();
-      const uint32_t cand = stage_rows(sm, nm, W, Fl, ~Vv);
+      const uint32_t cand = stage_rows<NARROW>(sm, nm, W, rl, Fl, ~Vv);
       if (bytes) nbytes += 4ull * W * (nm + 1);
       const uint32_t cw = __ballot_sync(0xffffffffu, cand != 0u);
       if (!cw) continue;
@@ -554,6 +597,7 @@ __global__ void __launch_bounds__(LVL_WARPS * 32, MFBC_PAIR_MIN_BLOCKS) k_lvl_fw
 // Every level-l quad of a single-item row gets a segment (its columns are
 // finalised by the gather even without successors); multi-item rows only emit
 // quads with pairs (their finalisation is k_lvl_hub_final).
+template <bool NARROW>
 __global__ void __launch_bounds__(LVL_WARPS * 32, MFBC_PAIR_MIN_BLOCKS) k_lvl_bwd_pairs(
     int64_t ib, int64_t ie, const int32_t* __restrict__ item_v, const int64_t* __restrict__ item_meta,
     const int32_t* __restrict__ col, int W, const uint32_t* __restrict__ Fl, const uint32_t* __restrict__ mem_l,
@@ -565,6 +609,7 @@ __global__ void __launch_bounds__(LVL_WARPS * 32, MFBC_PAIR_MIN_BLOCKS) k_lvl_bw
   const unsigned lane = lane_id();
   const uint32_t lt = (1u << lane) - 1u;
   const int Q = W / 4;
+  const RowLanes rl(W);
   unsigned long long nbytes = 0, npairs = 0;
   SlotCursor cur;
   if (*((volatile const uint32_t*)flags) & FLAG_ROUND_ABORT) return;
@@ -615,7 +660,7 @@ __global__ void __launch_bounds__(LVL_WARPS * 32, MFBC_PAIR_MIN_BLOCKS) k_lvl_bw
       const int nm = __popc(mm);
       if (isMem) sm.su[__popc(mm & lt)] = u;
       __syncwarp();
-      const uint32_t any = stage_rows(sm, nm, W, Fn, Fv);
+      const uint32_t any = stage_rows<NARROW>(sm, nm, W, rl, Fn, Fv);
       if (bytes) nbytes += 4ull * W * (nm + 1);
       const uint32_t words = __ballot_sync(0xffffffffu, multi ? any != 0u : Fv != 0u);
       if (words) emit_quads(sm, nm, v, multi, quads_of_words(words, Q), Q, hot, prow, pmask, segs, work, pair_cap,
@@ -1212,8 +1257,10 @@ __global__ void __launch_bounds__(256) k_lvl_output(int levels, int W, int nb, i
 static void set_smem_attrs() {
   static bool done = false;
   if (done) return;
-  cudaFuncSetAttribute(k_lvl_fwd_pairs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LVL_SMEM);
-  cudaFuncSetAttribute(k_lvl_bwd_pairs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LVL_SMEM);
+  cudaFuncSetAttribute(k_lvl_fwd_pairs<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LVL_SMEM);
+  cudaFuncSetAttribute(k_lvl_fwd_pairs<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LVL_SMEM);
+  cudaFuncSetAttribute(k_lvl_bwd_pairs<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LVL_SMEM);
+  cudaFuncSetAttribute(k_lvl_bwd_pairs<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LVL_SMEM);
   done = true;
 }
 
@@ -1298,14 +1345,15 @@ static mfbc_status level_round(RunCtx& rc, LevelState& s, bool fwd, int l, int64
   // priorities of the MFBr gather, whose rows' bit 31 the pair kernel sets
   const bool large = (uint64_t)items * (uint64_t)Qn >= 8ull * 32 * 4 * (fwd ? kGatherGrid : kBwdGatherGrid) * 8;
   const uint32_t* hot = large && !fwd && (uint64_t)n * (uint64_t)Qn < (1ull << 31) ? g.hot : nullptr;
+  const bool narrow = W <= NARROW_W;
   if (fwd)
-    PROF(K_LVL_FWD, (k_lvl_fwd_pairs<<<pgrid, LVL_WARPS * 32, LVL_SMEM, st>>>(
+    PROF(K_LVL_FWD, ((narrow ? k_lvl_fwd_pairs<true> : k_lvl_fwd_pairs<false>)<<<pgrid, LVL_WARPS * 32, LVL_SMEM, st>>>(
                         ib, ie, g.items_in.v, g.items_in.beg, g.col_t, W, s.full, s.V, Fl, Ml, Fn, Mn,
                         s.lists, &s.ctr->fwd_off, &s.ctr->list_count[0], s.list_cap, &s.ctr->flags,
                         &s.ctr->list_count[2], s.prow, s.pmask, s.segs, s.ctr->work, pair_cap, seg_cap, hot,
                         B ? B + K_LVL_FWD : nullptr, s.ctr->stat, ig, seg_chunk)));
   else
-    PROF(K_LVL_BWD, (k_lvl_bwd_pairs<<<pgrid, LVL_WARPS * 32, LVL_SMEM, st>>>(
+    PROF(K_LVL_BWD, ((narrow ? k_lvl_bwd_pairs<true> : k_lvl_bwd_pairs<false>)<<<pgrid, LVL_WARPS * 32, LVL_SMEM, st>>>(
                         ib, ie, g.items_out.v, g.items_out.beg, g.col, W, Fl, Ml, Fn, Mn,
                         &s.ctr->list_count[2], s.prow, s.pmask, s.segs, s.ctr->work, pair_cap, seg_cap, hot,
                         B ? B + K_LVL_BWD : nullptr, s.ctr->stat, ig, &s.ctr->flags, seg_chunk)));
