@@ -266,7 +266,7 @@ typedef struct {
  * int32[nsrc] for each candidate configuration and keeps the fastest on the
  * graph handle.  Candidates: n_b in {128, 256, 512, 1024} on the level kernels
  * and, for unit-weight graphs of at most 2^15 vertices and 2^19 arcs, n_b in
- * {32, 64, 128, 256} on the persistent small-graph kernel (AUTO itself takes
+ * {32, 64, 128, 256} on the small-graph family (AUTO itself takes
  * it up to 2^13 vertices and 2^18 arcs);
  * n_b in {128, 256, 512, 1024, 2048, 4096} on the general kernels (x the
  * atomic accumulator walking 1 or 8 arcs per step, the segmented accumulator,

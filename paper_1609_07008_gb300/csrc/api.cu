@@ -22,7 +22,7 @@ struct mfbc_graph {
   // autotuner results (mfbc_autotune): batch width per kernel family
   // (0 = not tuned), the family AUTO picks, and the general kernels' arcs
   // per step (0 = by average degree); force_arcs overrides it while tuning
-  int tuned_nb[4] = {0, 0, 0, 0};   // level, general, distance, persistent small-graph kernels
+  int tuned_nb[4] = {0, 0, 0, 0};   // level, general, distance, small-graph family
   int tuned_arcs = 0;
   int tuned_path = 0;               // kernel family for MFBC_PATH_AUTO (0 = by weights)
   int force_arcs = 0;
@@ -208,6 +208,7 @@ struct Plan {
   bool by_source = false;          // the call runs on the source kernel (source.cu):
   SourcePlan src, wide;            //   its blocks and state, and its redo form
   int redo_cap = 0;                //   sources a launch may hand to the redo form
+  int copies = 0;                  //   partial sums of lambda (one row per so many blocks)
   int groups = 0;                  // persistent small-graph kernel: block groups
   int64_t table_batches = 1;       //   and the batches its table holds
   int Lcap = 0;
@@ -245,14 +246,16 @@ static void level_caps(const DevGraph& g, int nb, int* Lcap, int64_t* list_cap) 
 // keeps narrow distances or counts, room for a list of redone sources and for
 // the wide form (with as many blocks as fit) in the same memory.  most: at most
 // this many blocks (0: as planned).
-static void source_sizes(const DevGraph& g, bool unit, int cols, int32_t nsrc, int most, Plan* p) {
+static void source_sizes(const DevGraph& g, bool unit, int cols, int32_t nsrc, int mode, int most, Plan* p) {
   source_plan(g, cols, unit, false, p->src);
   source_plan(g, cols, unit, true, p->wide);
   if (most > 0) p->src.slots = std::min(p->src.slots, most);
   p->redo_cap = p->src.unit || p->src.dm != p->wide.dm ? nsrc : 0;
   const size_t have = p->src.slot_bytes * (size_t)p->src.slots;
   p->wide.slots = (int)std::max<size_t>(1, std::min<size_t>((size_t)p->wide.slots, have / p->wide.slot_bytes));
-  p->state_bytes = std::max(source_bytes(p->src, p->redo_cap), source_bytes(p->wide, p->redo_cap));
+  p->copies = mode == 0 ? source_copies(p->src, g.n) : 0;
+  const size_t lam = (size_t)p->copies * g.n;
+  p->state_bytes = std::max(source_bytes(p->src, p->redo_cap, lam), source_bytes(p->wide, p->redo_cap, lam));
 }
 
 static size_t plan_bytes(const DevGraph& g, int path, int nb, int32_t nsrc, int mode, bool host_io,
@@ -264,7 +267,7 @@ static size_t plan_bytes(const DevGraph& g, int path, int nb, int32_t nsrc, int 
     // (on the unit-weight path n_b does not bound the sources in flight: a
     // block's state is small, and the blocks share nothing)
     const bool unit = path == MFBC_PATH_SMALL || path == MFBC_PATH_LEVEL;
-    source_sizes(g, unit, unit ? std::max(nsrc, 1) : std::min(nb, std::max(nsrc, 1)), nsrc, most, p);
+    source_sizes(g, unit, unit ? std::max(nsrc, 1) : std::min(nb, std::max(nsrc, 1)), nsrc, mode, most, p);
   } else if (path == MFBC_PATH_LEVEL) {
     level_caps(g, nb, &p->Lcap, &p->list_cap);
     // room for the general kernels at n_b = 32 too: the fallback used when
@@ -288,21 +291,20 @@ static size_t plan_bytes(const DevGraph& g, int path, int nb, int32_t nsrc, int 
 }
 
 // Kernel family for MFBC_PATH_AUTO without tuning: level kernels for unit
-// weights; distance-ordered kernels for weights <= 128 on graphs without hubs
-// (no degree above max(64, 4x the average): each distance step waits for its
-// longest adjacency list, so hubs make the steps slow -- weighted R-MAT 16,
-// 4096 sources: 3661 ms against 281 ms on the general kernels -- while grids
-// and uniform random graphs gain: weighted 256^2 grid 313 against 2883 ms,
-// Erdos-Renyi n = 2^16, k = 1024, 256 sources 153 against 326 ms); general
-// kernels otherwise.
-// Unit-weight graphs small enough for the persistent kernel to win: its
-// levels scan every (vertex, word) and every in-arc of an open vertex, which
-// costs more than the per-product kernels as the graph grows (R-MAT 14,
-// 16384 vertices, 4096 sources: 45 ms), while on small graphs the
-// per-product kernels wait on launches (Erdos-Renyi n = 1024, all sources:
-// 0.75 ms here against 14.7 ms).  mfbc_autotune compares the two.
+// weights; distance order for weights <= 128 on graphs without hubs (no degree
+// above max(64, 4x the average)); general kernels otherwise.  Within a family
+// the source kernel may run the call (the rules below).  Where the distance
+// kernels do, each step waits for its longest adjacency list, so hubs make the
+// steps slow (weighted R-MAT 16, 4096 sources: 3661 ms against 281 ms of the
+// general products), while uniform graphs gain (n = 2^16, k = 1024, 256 sources
+// 153 against 326 ms).
+// Unit-weight graphs small enough for one block per source whatever the number
+// of sources: level / source kernel, ms: R-MAT 13 (2.0 * 10^5 arcs), 1 / 456 / 1000
+// / 4096 sources 0.72 / 0.34, 1.19 / 1.02, 1.46 / 1.72, 5.99 / 5.84; R-MAT 12 0.57 /
+// 0.25, 0.92 / 0.52, 1.11 / 1.19; R-MAT 14 (4.3 * 10^5), 1000 / 4096 sources 2.2 /
+// 3.3, 8.0 / 11.7.  mfbc_autotune compares the families.
 static bool small_graph(const DevGraph& g) { return g.n <= (1 << 13) && g.nnz <= (1 << 18); }
-// graphs on which mfbc_autotune also times the persistent kernel
+// graphs on which mfbc_autotune also times the small-graph family
 static bool small_tunable(const DevGraph& g) { return g.n <= (1 << 15) && g.nnz <= (1 << 19); }
 
 static bool has_hubs(const DevGraph& g) {
@@ -804,8 +806,9 @@ mfbc_status source_path(Run& R, RunCtx& rc, const int32_t* d_src, int32_t nsrc, 
   const KId id = P.src.unit ? K_SMALL : K_DP_FWD;
   SourceState ss, sw;
   Carver c1(R.ws, R.ws_bytes), c2(R.ws, R.ws_bytes);
-  source_carve(c1, P.src, P.redo_cap, ss);
-  source_carve(c2, P.wide, P.redo_cap, sw);  // the same counters and list, other block states
+  const size_t copied = (size_t)P.copies * g.n;
+  source_carve(c1, P.src, P.redo_cap, copied, ss);
+  source_carve(c2, P.wide, P.redo_cap, copied, sw);  // the same counters and list, other block states
   std::vector<int32_t> rows;
   if (mode == 2 && nsrc) {
     rows.reserve((size_t)nsrc);
@@ -823,7 +826,8 @@ mfbc_status source_path(Run& R, RunCtx& rc, const int32_t* d_src, int32_t nsrc, 
     int32_t* dd = mode != 1 ? nullptr : staged ? stage_d : dist_out;
     double* ds = mode != 1 || !sigma_out ? nullptr : staged ? stage_s : sigma_out;
     double* lam = mode == 1 ? nullptr : d_lambda;
-    mfbc_status s = source_run(rc, P.src, ss, d_src + b0, mode == 2 ? d_row : nullptr, nullptr, na, lam, dd, ds, id);
+    mfbc_status s = source_run(rc, P.src, ss, d_src + b0, mode == 2 ? d_row : nullptr, nullptr, na, lam, P.copies, dd, ds,
+                               id);
     if (s) return s;
     for (bool again = true; again;) {
       MFBC_CUDA_TRY(cudaMemcpyAsync(h, ss.ctl, sizeof(SrcCtl), cudaMemcpyDeviceToHost, R.st), rc.err);
@@ -832,8 +836,8 @@ mfbc_status source_path(Run& R, RunCtx& rc, const int32_t* d_src, int32_t nsrc, 
       again = h->nredo != 0;                 // the wide form lists none
       if (!again) break;
       MFBC_CUDA_TRY(cudaMemsetAsync(&ss.ctl->nredo, 0, sizeof(uint32_t), R.st), rc.err);
-      s = source_run(rc, P.wide, sw, d_src + b0, mode == 2 ? d_row : nullptr, ss.redo, (int32_t)h->nredo, lam, dd, ds,
-                     id);
+      s = source_run(rc, P.wide, sw, d_src + b0, mode == 2 ? d_row : nullptr, ss.redo, (int32_t)h->nredo, lam,
+                     P.copies, dd, ds, id);
       if (s) return s;
     }
     if (staged) {
@@ -873,7 +877,7 @@ mfbc_status run(mfbc_graph* G, const int32_t* d_src, int32_t nsrc, int mode, dou
   SourceState srcs;
   Counters* ctr;
   SmallState ss;
-  if (P.by_source) { source_carve(c, P.src, P.redo_cap, srcs); ctr = srcs.ctr; }
+  if (P.by_source) { source_carve(c, P.src, P.redo_cap, (size_t)P.copies * g.n, srcs); ctr = srcs.ctr; }
   else if (P.path == MFBC_PATH_LEVEL) { level_carve(c, g, nb, P.Lcap, P.list_cap, ls); ctr = ls.ctr; }
   else if (P.path == MFBC_PATH_DIST) { dist_carve(c, g.n, nb, g.wmax + 1, ds); ctr = ds.ctr; }
   else if (P.path == MFBC_PATH_SMALL) { small_carve(c, g.n, nb, P.groups, ss); ctr = ss.ctr; }
@@ -1159,8 +1163,8 @@ mfbc_status entry(const mfbc_graph* Gc, const int32_t* sources, int32_t nsrc, in
     }
     d_src = ds;
   } else if (nsrc > 0 && R.plan.path != MFBC_PATH_SMALL) {
-    // device sources: validate the range on the host copy (the persistent
-    // small-graph path checks them on the device, without a round trip)
+    // device sources: validate the range on the host copy (the
+    // small-graph family checks them on the device, without a round trip)
     std::vector<int32_t> hs((size_t)nsrc);
     if (cudaMemcpyAsync(hs.data(), sources, sizeof(int32_t) * (size_t)nsrc, cudaMemcpyDeviceToHost, R.st) != cudaSuccess ||
         cudaStreamSynchronize(R.st) != cudaSuccess) {

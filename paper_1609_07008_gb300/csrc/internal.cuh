@@ -239,6 +239,7 @@ struct SrcCtl {          // read back once per call
   uint32_t flags;        // FLAG_* bits
 };
 struct SourceState {
+  double* lam;           // [copies][n] partial sums of lambda (calls with one lambda row)
   char* slots;           // [slots] block states of slot_bytes
   SrcCtl* ctl;
   int32_t* redo;         // sources for the wide form
@@ -248,8 +249,10 @@ struct SourceState {
 // 64-bit counts; wide: the form without narrow distances or counts, which
 // sources that outgrow them are redone in.
 void source_plan(const DevGraph& g, int cols, bool unit, bool wide, SourcePlan& p);
-size_t source_bytes(const SourcePlan& p, int32_t nredo);
-void source_carve(Carver& c, const SourcePlan& p, int32_t nredo, SourceState& s);
+// copies of lambda that the blocks of a call with one lambda row add into (0: none)
+int source_copies(const SourcePlan& p, int32_t n);
+size_t source_bytes(const SourcePlan& p, int32_t nredo, size_t lam);   // lam = copies * n
+void source_carve(Carver& c, const SourcePlan& p, int32_t nredo, size_t lam, SourceState& s);
 
 // Persistent path for small unit-weight graphs: whole batches inside one
 // cooperative launch, block groups taking batches from a device queue.  See
@@ -325,9 +328,9 @@ mfbc_status dist_output(RunCtx& rc, DistState& s, int nactive, int32_t* dist_out
 // The sources d_src[0 .. nsrc) -- or, with d_list, d_src[d_list[0 .. nsrc)] --
 // on the source kernel, launched once and not waited for.  d_row: lambda row of
 // each source or null (row 0).  lambda null: MFBF only, source i writing row i
-// of dist_out / sigma_out.
+// of dist_out / sigma_out.  copies: as carved (d_row null).
 mfbc_status source_run(RunCtx& rc, const SourcePlan& p, SourceState& s, const int32_t* d_src, const int32_t* d_row,
-                       const int32_t* d_list, int32_t nsrc, double* lambda, int32_t* dist_out, double* sigma_out,
+                       const int32_t* d_list, int32_t nsrc, double* lambda, int copies, int32_t* dist_out, double* sigma_out,
                        KId id);
 
 // All batches of a call on the persistent small-graph kernel.  d_src_all:
