@@ -1020,7 +1020,9 @@ mfbc_status source_run(RunCtx& rc, const SourcePlan& p, SourceState& s, const in
   a.redo = s.redo;
   a.bytes = rc.prof->count_bytes ? &s.ctr->bytes[id] : nullptr;
   const void* k = src_kernel(p, !g.directed);
-  MFBC_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem), rc.err);
+  // (the limit is the kernel's, not the launch's: calls on other threads must not
+  // lower it between here and the launch)
+  MFBC_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SRC_SMEM_MAX), rc.err);
   MFBC_CUDA_TRY(cudaMemsetAsync(&s.ctl->head, 0, sizeof(uint32_t), rc.stream), rc.err);
   if (lambda && copies)
     MFBC_CUDA_TRY(cudaMemsetAsync(s.lam, 0, sizeof(double) * (size_t)copies * g.n, rc.stream), rc.err);

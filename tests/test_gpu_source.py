@@ -181,3 +181,36 @@ def test_workspaces_of_any_accepted_size():
     close(G.bc(srcs, workspace=narrow, n_b=32), want)
     close(G.bc(srcs, workspace=narrow), want)
     G.close()
+
+
+def test_threads_with_different_shared_memory_sizes():
+    # one kernel form, two graphs whose blocks take different amounts of shared
+    # memory, called from threads at the same time
+    import threading
+    import torch
+    jobs = []
+    for n, seed in ((300, 30), (3001, 31), (9001, 32), (16384, 33)):
+        g = gg.erdos_renyi(n, 12, seed=seed)
+        srcs = gg.sample_sources(g, 40, seed=1)
+        jobs.append((mfbc.Graph.from_csr(g), torch.from_numpy(srcs).cuda(), oracle.bc(g, srcs)))
+    failed = []
+
+    def work(G, srcs, want):
+        try:
+            stream = torch.cuda.Stream()
+            for _ in range(200):
+                with torch.cuda.stream(stream):
+                    lam = G.bc(srcs, stream=stream)
+            stream.synchronize()
+            close(lam.cpu().numpy(), want)
+        except BaseException as e:
+            failed.append(e)
+
+    threads = [threading.Thread(target=work, args=j) for j in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed, failed[0]
+    for G, _, _ in jobs:
+        G.close()
