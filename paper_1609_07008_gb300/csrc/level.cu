@@ -1200,9 +1200,9 @@ __global__ void k_lvl_clear_rows(ClearSpan c, int W, uint32_t* F, size_t level_w
 // vertex-major state and the source-major rows are touched in whole lines.  A
 // warp reads one vertex's mask word of every level (all lanes the same word; the
 // sector's other words are for the blocks beside it and come from the L2).
-// Bound by the bit tests and the stores (12 bytes per pair).  R-MAT 18, 300 sources (0.94 GB of
-// rows): 3.0 -> 0.47 ms against a fill of the rows and a scatter of 12 bytes per
-// pair over n-strided rows.
+// Bound by the bit tests and the stores (12 bytes per pair).  R-MAT 18, 300
+// sources (0.94 GB of rows): 3.0 -> 0.47 ms against a fill of the rows and a
+// scatter of 12 bytes per pair over n-strided rows.
 __global__ void __launch_bounds__(256) k_lvl_output(int levels, int W, int nb, int nactive, int32_t n,
                                                     const uint32_t* __restrict__ F, const uint64_t* __restrict__ sv,
                                                     int32_t* dist_out, double* sigma_out) {
