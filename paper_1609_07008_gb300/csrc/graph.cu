@@ -124,6 +124,23 @@ static mfbc_status dev_alloc(DevGraph* g, T** p, size_t count, std::string* err)
     if (_s != MFBC_OK) return _s; \
   } while (0)
 
+// Columns and, weighted, weights and packed arcs (see pack_arcs).  Up to
+// JOINED_ARCS arcs they share one allocation, whose calls are what creating a
+// small weighted graph spends most on; beyond, packed arcs are allocated only
+// once the weights are known to differ from 1.
+constexpr int64_t JOINED_ARCS = 1 << 22;
+static mfbc_status alloc_arcs(DevGraph* g, bool weighted, int32_t** col, int32_t** w, uint32_t** pk, std::string* err) {
+  const size_t nnz = (size_t)g->nnz, stride = (nnz + 63) & ~(size_t)63;
+  if (!weighted || g->nnz > JOINED_ARCS) {
+    TRY(dev_alloc(g, col, nnz, err));
+    return weighted ? dev_alloc(g, w, nnz, err) : MFBC_OK;
+  }
+  TRY(dev_alloc(g, col, 3 * stride, err));
+  *w = *col + stride;
+  *pk = reinterpret_cast<uint32_t*>(*col + 2 * stride);
+  return MFBC_OK;
+}
+
 // empty_rows: give every row without arcs one empty item.  The MFBr gather
 // must visit DAG sinks too (their frontier value 1/sigma_bar is written by
 // that visit); in an undirected graph a vertex without arcs can only be a
@@ -209,11 +226,11 @@ static mfbc_status pack_arcs(DevGraph* g, cudaStream_t st, std::string* err) {
   if (cb + wb > 32) { *err = "column and weight of an arc do not fit in 32 bits"; return MFBC_ERR_OVERFLOW; }
   g->pk_bits = cb;
   const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>((g->nnz + 255) / 256, 152 * 16));
-  TRY(dev_alloc(g, &g->pk, (size_t)g->nnz, err));
+  if (!g->pk) TRY(dev_alloc(g, &g->pk, (size_t)g->nnz, err));
   k_pack_arcs<<<blocks, 256, 0, st>>>(g->col, g->w, g->nnz, cb, g->pk);
-  g->pk_t = g->pk;
-  if (g->directed) {
-    TRY(dev_alloc(g, &g->pk_t, (size_t)g->nnz, err));
+  if (!g->directed) g->pk_t = g->pk;
+  else {
+    if (!g->pk_t) TRY(dev_alloc(g, &g->pk_t, (size_t)g->nnz, err));
     k_pack_arcs<<<blocks, 256, 0, st>>>(g->col_t, g->w_t, g->nnz, cb, g->pk_t);
   }
   return MFBC_OK;
@@ -444,8 +461,7 @@ mfbc_status graph_build(int32_t n, int64_t nnz, const int64_t* h_rowptr, const i
   g->nnz = nnz;
   g->directed = !(flags & MFBC_UNDIRECTED);
   TRY(dev_alloc(g, &g->rowptr, (size_t)n + 1, err));
-  TRY(dev_alloc(g, &g->col, (size_t)nnz, err));
-  if (h_w) TRY(dev_alloc(g, &g->w, (size_t)nnz, err));
+  TRY(alloc_arcs(g, h_w != nullptr, &g->col, &g->w, &g->pk, err));
   ValFlags* d_f;
   TRY(dev_alloc(g, &d_f, 1, err));
   MFBC_CUDA_TRY(cudaMemcpyAsync(g->rowptr, h_rowptr, sizeof(int64_t) * ((size_t)n + 1), cudaMemcpyHostToDevice, st), err);
@@ -532,7 +548,7 @@ mfbc_status graph_build(int32_t n, int64_t nnz, const int64_t* h_rowptr, const i
     return MFBC_ERR_OVERFLOW;
   }
   g->unit = !f.non_unit;
-  if (g->unit && g->w) { g->w = nullptr; }   // all ones: treat as unweighted (array still owned)
+  if (g->unit && g->w) { g->w = nullptr; g->pk = nullptr; }   // all ones: treat as unweighted (arrays still owned)
   if (g->directed) {
     // A^T by a stable counting sort on the host: rows of A^T are sorted by
     // source vertex, so the transposed graph is deterministic.
@@ -551,8 +567,7 @@ mfbc_status graph_build(int32_t n, int64_t nnz, const int64_t* h_rowptr, const i
         if (g->w) wtv[p] = h_w[k];
       }
     TRY(dev_alloc(g, &g->rowptr_t, (size_t)n + 1, err));
-    TRY(dev_alloc(g, &g->col_t, (size_t)nnz, err));
-    if (g->w) TRY(dev_alloc(g, &g->w_t, (size_t)nnz, err));
+    TRY(alloc_arcs(g, g->w != nullptr, &g->col_t, &g->w_t, &g->pk_t, err));
     MFBC_CUDA_TRY(cudaMemcpyAsync(g->rowptr_t, rpt.data(), sizeof(int64_t) * rpt.size(), cudaMemcpyHostToDevice, st), err);
     if (nnz) MFBC_CUDA_TRY(cudaMemcpyAsync(g->col_t, ct.data(), sizeof(int32_t) * ct.size(), cudaMemcpyHostToDevice, st), err);
     if (g->w && nnz) MFBC_CUDA_TRY(cudaMemcpyAsync(g->w_t, wtv.data(), sizeof(int32_t) * wtv.size(), cudaMemcpyHostToDevice, st), err);
