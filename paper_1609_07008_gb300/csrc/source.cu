@@ -118,6 +118,11 @@ struct SrcArgs {
 // A vertex's reduction in one step, kept in 8 bytes of shared memory: FP64 sums
 // (values, and path counts of weighted graphs: integers below 2^53, exact in any
 // order) or exact 64-bit counts (unit weights).
+// Counts of 2^58 send the source to the FP64 form, and every sum is looked at as
+// it grows, not only when it is complete: a vertex with more than 64 predecessors
+// of almost 2^58 paths each could pass 2^64 and come back small.  The counts that
+// a batch of 32 arcs or a piece of a hub row adds are below 2^58 each, so no sum
+// wraps before one of at least 2^58 was seen.
 struct SumF64 {
   double s = 0.0;
   __device__ __forceinline__ static SumF64 of_count(uint64_t x) { return {__longlong_as_double((long long)x)}; }
@@ -125,6 +130,7 @@ struct SumF64 {
   __device__ __forceinline__ static uint64_t one() { return (uint64_t)__double_as_longlong(1.0); }
   __device__ __forceinline__ uint64_t bits() const { return (uint64_t)__double_as_longlong(s); }
   __device__ __forceinline__ void add(const SumF64& o) { s += o.s; }
+  __device__ __forceinline__ bool wide() const { return false; }
   __device__ __forceinline__ SumF64 up(int o) const { return {__shfl_up_sync(0xffffffffu, s, o)}; }
 };
 struct SumU64 {
@@ -133,6 +139,7 @@ struct SumU64 {
   __device__ __forceinline__ static uint64_t one() { return 1ull; }
   __device__ __forceinline__ uint64_t bits() const { return i; }
   __device__ __forceinline__ void add(const SumU64& o) { i += o.i; }
+  __device__ __forceinline__ bool wide() const { return i >= (1ull << 58); }
   __device__ __forceinline__ SumU64 up(int o) const { return {__shfl_up_sync(0xffffffffu, i, o)}; }
 };
 template <int ILP>
@@ -251,6 +258,7 @@ __device__ __forceinline__ void src_flush(const SrcArgs& a, SrcWarp<ILP>& wb, S&
     else sum = Sum::of_value(wb.acc[t]);
     sum.add(x);
     wb.acc[t] = sum.bits();
+    if (sum.wide()) st.sh.redo = 1u;
   }
   __syncwarp();
 }
@@ -434,8 +442,7 @@ __device__ __forceinline__ double src_sigma(uint64_t sv) {
   return UNIT ? (double)sv : __longlong_as_double((long long)sv);
 }
 // sigma_bar of a settled vertex: stored beside a zeta of 0, and checked against
-// 2^53 (FP64 output inexact) and, for 64-bit counts, 2^58 (later sums could
-// wrap: the source is redone in FP64).
+// 2^53 (FP64 output inexact).
 __device__ __forceinline__ void src_put(SrcCell* c, uint64_t sv) {
   *reinterpret_cast<ulonglong2*>(c) = make_ulonglong2(sv, 0ull);
 }
@@ -447,10 +454,7 @@ __device__ __forceinline__ void src_put_count(const SrcArgs& a, S& st, int32_t v
 template <class S>
 __device__ __forceinline__ void src_put_count(const SrcArgs& a, S& st, int32_t v, const SumU64& x) {
   src_put(&st.cell[v], x.i);
-  if (x.i >= (1ull << 53)) {
-    atomicOr(&a.ctl->flags, FLAG_SIGMA_INEXACT);
-    if (x.i >= (1ull << 58)) st.sh.redo = 1u;
-  }
+  if (x.i >= (1ull << 53)) atomicOr(&a.ctl->flags, FLAG_SIGMA_INEXACT);
 }
 // zeta of a vertex (pulled form): its lambda term, and the value zeta +
 // 1/sigma_bar in the place of the count.
@@ -463,8 +467,9 @@ __device__ __forceinline__ void src_put_value(SrcCell* c, double* lam, const Sum
 
 // Hub rows: a warp's share of the row's sum joins the total; the total read back.
 __device__ __forceinline__ void src_hub_add(SrcShared& sh, int h, const SumF64& x) { atomicAdd(&sh.hacc[h], x.s); }
-__device__ __forceinline__ void src_hub_add(SrcShared& sh, int h, const SumU64& x) {
-  atomicAdd(&sh.hcnt[h], (unsigned long long)x.i);
+__device__ __forceinline__ void src_hub_add(SrcShared& sh, int h, SumU64 x) {
+  x.add(SumU64{atomicAdd(&sh.hcnt[h], (unsigned long long)x.i)});
+  if (x.wide()) sh.redo = 1u;
 }
 __device__ __forceinline__ void src_hub_get(const SrcShared& sh, int h, SumF64& x) { x.s = sh.hacc[h]; }
 __device__ __forceinline__ void src_hub_get(const SrcShared& sh, int h, SumU64& x) { x.i = sh.hcnt[h]; }
