@@ -56,11 +56,11 @@
 
 #include "dfloat.cuh"
 #include "internal.cuh"
+#include "pieces.h"
 
 namespace mfbc {
 
-constexpr int SRC_HUB_ARCS = 512;      // longer rows are cut into pieces for the block's warps
-constexpr int SRC_PIECE = 256;         // arcs of a piece
+constexpr int SRC_HUB_ARCS = 512;      // longer rows are cut into pieces (pieces.h) for the block's warps
 constexpr int SRC_HUBS = 64;           // such rows a step can list (more are walked by their own warp)
 constexpr int SRC_BIG_ARCS = 64;       // rows from here on are walked whole, shorter ones as one flat list
 constexpr int SRC_SMEM_MAX = 226 * 1024;
@@ -485,7 +485,6 @@ __device__ __forceinline__ bool src_list_hub(SrcShared& sh, int32_t v, uint32_t 
   sh.hcnt[h] = 0ull;
   return true;
 }
-__device__ __forceinline__ uint32_t src_pieces(int32_t len) { return (uint32_t)((len + SRC_PIECE - 1) / SRC_PIECE); }
 // The hub row that piece p belongs to: the last of the nh listed rows whose
 // first piece is at most p (whole warp).
 __device__ __forceinline__ uint32_t src_piece_row(const SrcShared& sh, uint32_t nh, uint32_t p) {
@@ -643,23 +642,23 @@ __global__ void __launch_bounds__(1024) k_src_bc(SrcArgs a) {
         for (uint32_t p = (uint32_t)wid; p < np; p += (uint32_t)nwarp) {
           const uint32_t h = src_piece_row(sh, nh, p);
           const int32_t v = sh.hv[h];
-          const uint32_t i = p - sh.hbase[h];           // the row's piece: out-arcs first, then in-arcs
           const int64_t b = __ldg(&a.rp[v]);
           const int32_t len = (int32_t)(__ldg(&a.rp[v + 1]) - b);
-          const uint32_t po = src_pieces(len);
+          int64_t bt = 0;
+          int32_t lent = 0;
+          if (!SYM) {
+            bt = __ldg(&a.rpt[v]);
+            lent = (int32_t)(__ldg(&a.rpt[v + 1]) - bt);
+          }
+          const HubPiece hp = src_hub_piece(len, lent, p - sh.hbase[h]);
+          if (!hp.count) continue;                      // (pieces of a row not listed)
           if (lane == 0) wb.acc[0] = 0ull;
           cx.mv = v;
           __syncwarp();
-          if (i < po) {
-            const int32_t k0 = (int32_t)i * SRC_PIECE;
-            cx.template fwd<SYM, true, Cnt>(a.arc, b + k0, lane == 0 ? min(SRC_PIECE, len - k0) : 0, d, slot);
-          } else if (!SYM) {
-            const int64_t bt = __ldg(&a.rpt[v]);
-            const int32_t lent = (int32_t)(__ldg(&a.rpt[v + 1]) - bt);
-            const int32_t k0 = (int32_t)(i - po) * SRC_PIECE;      // (pieces of a row not listed: past its end)
-            if (k0 < lent)
-              cx.template fwd<true, false, Cnt>(a.arct, bt + k0, lane == 0 ? min(SRC_PIECE, lent - k0) : 0, d, slot);
-          }
+          if (!hp.in)
+            cx.template fwd<SYM, true, Cnt>(a.arc, b + hp.first, lane == 0 ? hp.count : 0, d, slot);
+          else if (!SYM)
+            cx.template fwd<true, false, Cnt>(a.arct, bt + hp.first, lane == 0 ? hp.count : 0, d, slot);
           cx.template drain<Cnt, true>(true);
           __syncwarp();
           if (lane == 0 && wb.acc[0]) src_hub_add(sh, (int)h, Cnt::of_count(wb.acc[0]));
@@ -833,11 +832,11 @@ __global__ void __launch_bounds__(1024) k_src_bc(SrcArgs a) {
           const int32_t v = sh.hv[h];
           const int64_t b = __ldg(&a.rp[v]);
           const int32_t len = (int32_t)(__ldg(&a.rp[v + 1]) - b);
-          const int32_t k0 = (int32_t)(p - sh.hbase[h]) * SRC_PIECE;
-          if (k0 >= len) continue;                      // (pieces of a row not listed)
+          const HubPiece hp = src_hub_piece(len, 0, p - sh.hbase[h]);
+          if (!hp.count) continue;                      // (pieces of a row not listed)
           if (lane == 0) wb.acc[0] = 0ull;
           __syncwarp();
-          cx.template bwd<Val>(b + k0, lane == 0 ? min(SRC_PIECE, len - k0) : 0, st.tau(v));
+          cx.template bwd<Val>(b + hp.first, lane == 0 ? hp.count : 0, st.tau(v));
           cx.template drain<Val, false>(true);
           __syncwarp();
           if (lane == 0 && wb.acc[0]) src_hub_add(sh, (int)h, Val::of_value(wb.acc[0]));
