@@ -163,6 +163,10 @@ typedef struct {
                                     segment buffers of 2^16 slots, so their rounds overflow and
                                     are redone over halves of the work items (the path a graph
                                     beyond 2^31 pairs per round takes); results are unchanged */
+#define MFBC_OPT_TEST_FAMILY_KERNELS 32u  /* test hook: the kernels of the call's family (MFBC_PATH_*)
+                                    run it, not the one-block-per-source kernel that takes most
+                                    calls of the small, distance and, under AUTO, level and general
+                                    families; results are unchanged up to the order of sums */
 
 /* Build a device-resident graph from HOST compressed-row arrays (Sec. 2.1:
  * A(i,j) = w(i,j) for (i,j) in E; the paper's Tensor::write of the input,

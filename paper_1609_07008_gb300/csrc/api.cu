@@ -392,12 +392,13 @@ static mfbc_status make_plan(const mfbc_graph* G, int32_t nsrc, int mode, const 
     if (maxnb < 32) return fail(MFBC_ERR_INVALID, "MFBC_PATH_DIST needs n < 2^27");
   }
   // may the source kernel take the call, and does the rule choose it?
+  const bool hooked = opt && (opt->flags & MFBC_OPT_TEST_FAMILY_KERNELS);
   const bool open_general = path == MFBC_PATH_GENERAL && (!opt || (opt->path == MFBC_PATH_AUTO && !opt->accumulator)) &&
                             !G->tuned_path && !G->tuned_arcs && !G->tuned_accum && !G->force_arcs;
   const bool small = path == MFBC_PATH_SMALL && !(opt && (opt->flags & MFBC_OPT_TEST_STALL));
   const bool open_level = path == MFBC_PATH_LEVEL && !G->tuned_path && !G->tuned_nb[0] &&
                           (!opt || (opt->path == MFBC_PATH_AUTO && !(opt->flags & MFBC_OPT_TEST_SMALL_ROUNDS)));
-  const bool can_source = g.nnz < (1ll << 31) && (path == MFBC_PATH_DIST || small || (open_general && general_by_source(g, INT32_MAX)) ||
+  const bool can_source = !hooked && g.nnz < (1ll << 31) && (path == MFBC_PATH_DIST || small || (open_general && general_by_source(g, INT32_MAX)) ||
                                                   (open_level && level_by_source(g, 1)));
   const bool by_source = can_source && (small || (path == MFBC_PATH_DIST    ? dist_by_source(g, nsrc)
                                                   : path == MFBC_PATH_LEVEL ? level_by_source(g, nsrc)
