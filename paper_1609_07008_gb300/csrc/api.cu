@@ -1,6 +1,7 @@
 // C ABI of the MFBC library: argument checks, choice of kernel family and
 // batch width, scratch management, and the batch loop of Algorithm 3.
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <chrono>
 #include <mutex>
@@ -322,18 +323,53 @@ static int default_path(const DevGraph& g) {
 // kernels and for calls of the general kernels that leave the choice open
 // (MFBC_PATH_AUTO, untuned, no accumulator named).
 //
-// A source on one block takes about 4 us per distance value that occurs plus
-// its arcs' share, however few sources run.  The distance kernels spread a step
-// over the whole GPU, which wins where few sources meet wide steps: uniform
-// n = 300 000, k = 16, weights <= 20, 1 / 8 / 32 / 48 sources 10.3 / 10.9 / 12.3
-// / 13.2 ms here against 2.4 / 4.5 / 9.3 / 14.4 there; n = 10^6, k = 8: 25 / 29 /
-// 33 / 35 against 3.5 / 10 / 24 / 38; n = 100 000, k = 32, weights <= 100, 1 / 8
-// sources 6.0 / 6.1 against 5.2 / 6.6.  On lattices (degrees <= 8) the steps are
-// narrow and the blocks win from one source on: weighted 256^2 grid, 1 / 64 /
-// 256 sources 7.1 / 10.8 / 13 ms against 24 / 49 / 58.
+// A source on one block takes 3.3 us per distance value that occurs plus its
+// vertices' and arcs' share, however few sources run.  The distance kernels spread
+// a step over the whole GPU at 20-40 us a step (and the walk of its longest row),
+// which wins where few sources meet few wide steps.  Both sides in ms, source /
+// distance kernels, at 1, 8, 24, 40 sources:
+//   uniform n = 2^20, k = 6, weights <= 20     15 / 4.1, 17 / 11, 18 / 21, 20 / 34
+//                            weights <= 100    17 / 14, 20 / 21, 21 / 37, 22 / 54
+//           n = 2^18, k = 64, weights <= 20    15 / 2.4, 16 / 4.9, 16 / 7.6, 17 / 13
+//           n = 2^17, k = 64, weights <= 4     7.2 / 1.2, 7.3 / 1.9, 7.4 / 3.0, 7.5 / 4.9
+//           n = 2^16, k = 6, weights <= 100    2.2 / 7.9, 2.2 / 11, 2.2 / 13, 2.3 / 14
+//   three random permutations, weights <= 16, n = 2^20, 1 / 8 / 40 sources
+//                                              14 / 3.5, 16 / 8.6, 19 / 25
+//   weighted grid, 512^2, 1 / 8 / 64 sources   21 / 93, 21 / 94, 24 / 107
+//                  2048^2                      109 / 299, 124 / 397, 130 / 553
+// So the line is drawn by an estimate of both times.  Its coefficients were fitted
+// to 250 such pairs (n = 2^14 .. 2^22, k = 3 .. 1024, weights <= 4 .. 100); over
+// them the choice is at most 1.33 times slower than the better side, 1 % on
+// average.  Above 40 sources, and below 2^15 vertices, the blocks win or come
+// within 10 % throughout.
+static double distance_values(const DevGraph& g) {       // that a source meets, about
+  const double deg = std::max(1.0, (double)g.nnz / g.n);
+  // (without an estimate -- unit weights -- low degrees are taken for a lattice's)
+  const double hops = g.hops > 0.0 ? g.hops
+                      : std::max(g.max_deg, g.max_in_deg) <= 8 ? 0.7 * std::sqrt((double)g.n)
+                                                               : std::log((double)g.n) / std::log(std::max(2.0, deg));
+  return hops * (2.0 + 1.25 * g.wmax / std::sqrt(deg));
+}
+// us of the distance kernels for nsrc sources, nb at a time
+static double dist_steps_us(const DevGraph& g, int32_t nsrc, int nb) {
+  const double steps = distance_values(g), row = (double)std::max(g.max_deg, g.max_in_deg);
+  auto batch = [&](int k) {
+    return steps * (18.0 + 0.5 * std::min(k, 16) + row) + k * (0.55e-3 * g.n + 0.006e-3 * (double)g.nnz);
+  };
+  return nsrc / nb * batch(nb) + (nsrc % nb ? batch(nsrc % nb) : 0.0);
+}
+// us of the source kernel on weighted graphs, `blocks` sources at a time
+static double dist_source_us(const DevGraph& g, int32_t nsrc, int blocks) {
+  // (long rows are walked whole, and faster where tau is in shared memory)
+  const double arc = g.nnz < 128 * (int64_t)g.n ? 0.7e-3 : g.n > 100000 ? 0.55e-3 : 0.26e-3;
+  const double one = 3.3 * distance_values(g) + (13.5e-3 + 0.15e-3 * std::min({nsrc, blocks, 152})) * g.n +
+                     arc * (double)g.nnz;
+  return one * ((nsrc + blocks - 1) / blocks);
+}
 static bool dist_by_source(const DevGraph& g, int32_t nsrc) {
-  if (std::max(g.max_deg, g.max_in_deg) <= 8) return true;
-  return !((g.n >= (1 << 18) && nsrc <= 40) || (g.n >= (1 << 16) && nsrc <= 4));
+  if (g.n < (1 << 15) || nsrc > 40) return true;
+  const int32_t k = std::max(nsrc, 1);
+  return dist_source_us(g, k, k) < dist_steps_us(g, k, 64);
 }
 // The general kernels' time goes with their 15-25 Bellman-Ford products (0.1-0.3
 // ms each and up) whatever the weights are, the source kernel's with the

@@ -12,6 +12,7 @@
 // (OVERFLOW otherwise): every finite distance and every candidate tau + w of
 // the MFBF product then fits.
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 
 #include "internal.cuh"
@@ -234,6 +235,55 @@ static mfbc_status pack_arcs(DevGraph* g, cudaStream_t st, std::string* err) {
     k_pack_arcs<<<blocks, 256, 0, st>>>(g->col_t, g->w_t, g->nnz, cb, g->pk_t);
   }
   return MFBC_OK;
+}
+
+// About how many arcs the far ends of the graph are apart, from the breadth-first
+// ball of up to BALL vertices around a vertex of high degree.  A ball that needs
+// more levels than doubling would (with some room) grows like a power of its
+// radius, as on lattices and road networks, and is carried on with that power;
+// otherwise it grows by a factor a level.  Only api.cu's choice between kernels of
+// equal results depends on it, and only for graphs of HOPS_ROWS vertices and more.
+// It takes 40-80 us on the host.  (A ball of 4096 would tell three-dimensional
+// lattices from graphs of degree 2 that double, but takes 150-300 us.)
+constexpr int32_t HOPS_ROWS = 1 << 15;
+static double estimate_hops(int32_t n, const int64_t* rp, const int32_t* col, const std::vector<int32_t>& roots) {
+  constexpr int BALL = 1024, SLOTS = 4 * BALL, ARCS = 1 << 14;
+  const size_t target = BALL;
+  std::vector<int32_t> slots, order;
+  std::vector<size_t> size, best;      // vertices within l levels
+  for (size_t r = 0; r < std::min<size_t>(roots.size(), 4); r++) {       // (a root's component may be small)
+    slots.assign(SLOTS, -1);
+    order.clear();
+    size.clear();
+    auto visit = [&](int32_t v) {
+      uint32_t h = ((uint32_t)v * 2654435769u) >> 20;                     // 12 bits
+      while (slots[h] != v && slots[h] != -1) h = (h + 1) % SLOTS;
+      if (slots[h] == v) return;
+      slots[h] = v;
+      order.push_back(v);
+    };
+    visit(roots[r]);
+    size.push_back(1);
+    int64_t arcs = 0;
+    for (size_t at = 0; order.size() < target && arcs < ARCS && at < order.size();) {
+      for (const size_t end = order.size(); at < end && order.size() < target && arcs < ARCS; at++)
+        for (int64_t k = rp[order[at]]; k < rp[order[at] + 1] && order.size() < target && arcs < ARCS; k++, arcs++)
+          visit(col[k]);
+      if (order.size() > size.back()) size.push_back(order.size());
+    }
+    if (best.empty() || size.back() > best.back()) best = size;
+    if (best.back() >= target || arcs >= ARCS) break;
+  }
+  if (best.size() < 2) return 1.0;
+  const double L = (double)best.size() - 1.0, B = (double)best.back();
+  if (best.back() < target) return L;                                     // the whole component
+  if (L > 1.15 * std::log2(B)) {
+    const size_t half = best.size() / 2;
+    const double power = std::max(1.0, std::log(B / (double)best[half]) / std::log(L / (double)half));
+    return L * std::pow(n / B, 1.0 / power);
+  }
+  const double deg = std::max(2.0, (double)rp[n] / n), inner = (double)best[best.size() - 2];
+  return std::max(1.0, std::min(L, L - 1.0 + std::log(B / inner) / std::log(deg)) * std::log((double)n) / std::log(B));
 }
 
 // ------------------------------------------------- row structure on the device
@@ -548,6 +598,8 @@ mfbc_status graph_build(int32_t n, int64_t nnz, const int64_t* h_rowptr, const i
     return MFBC_ERR_OVERFLOW;
   }
   g->unit = !f.non_unit;
+  if (!g->unit && n >= HOPS_ROWS && g->wmax + 1 <= DIST_MAX_BUCKETS)
+    g->hops = estimate_hops(n, h_rowptr, h_col, g->landmarks);
   if (g->unit && g->w) { g->w = nullptr; g->pk = nullptr; }   // all ones: treat as unweighted (arrays still owned)
   if (g->directed) {
     // A^T by a stable counting sort on the host: rows of A^T are sorted by

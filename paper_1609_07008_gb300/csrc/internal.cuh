@@ -54,6 +54,7 @@ struct DevGraph {
   uint32_t* pk = nullptr;          // A's arcs as column | weight << pk_bits (nullptr when unit)
   uint32_t* pk_t = nullptr;        //   and those of A^T (aliases pk when undirected)
   int pk_bits = 0;
+  double hops = 0.0;               // weighted: estimated arcs across the graph (0: not estimated)
   ItemList items_in;               // over A^T rows (MFBF pull gathers in-arcs)
   ItemList items_out;              // over A rows   (MFBr pull gathers out-arcs)
   std::vector<void*> owned;        // device allocations to free
