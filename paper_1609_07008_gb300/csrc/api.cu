@@ -246,11 +246,11 @@ static void level_caps(const DevGraph& g, int nb, int* Lcap, int64_t* list_cap) 
 // The source kernel's blocks and state: its form for the graph and, when that
 // keeps narrow distances or counts, room for a list of redone sources and for
 // the wide form (with as many blocks as fit) in the same memory.  most: at most
-// this many blocks (0: as planned).
+// this many blocks, planned for as many sources (0: for `cols`).
 static void source_sizes(const DevGraph& g, bool unit, int cols, int32_t nsrc, int mode, int most, Plan* p) {
+  if (most > 0) cols = std::min(cols, most);
   source_plan(g, cols, unit, false, p->src);
   source_plan(g, cols, unit, true, p->wide);
-  if (most > 0) p->src.slots = std::min(p->src.slots, most);
   p->redo_cap = p->src.unit || p->src.dm != p->wide.dm ? nsrc : 0;
   const size_t have = p->src.slot_bytes * (size_t)p->src.slots;
   p->wide.slots = (int)std::max<size_t>(1, std::min<size_t>((size_t)p->wide.slots, have / p->wide.slot_bytes));
@@ -400,6 +400,30 @@ static bool level_by_source(const DevGraph& g, int32_t nsrc) {
          (nsrc <= 152 || (int64_t)nsrc * g.nnz <= 130000000);
 }
 
+// The rules above compare the sides at full width.  With little scratch, or a
+// narrow n_b, the source kernel is left with fewer blocks than there are SMs and
+// sources, while the family's kernels still use the whole device, nb columns at a
+// time; `blocks` sources at once against that, in ms, source / family:
+//   distances, uniform n = 100 000, k = 16, weights <= 20, 512 sources, with the
+//     scratch of 32 / 64 / 128 / 256 columns (5 / 10 / 20 / 40 blocks) 361 / 60,
+//     159 / 50, 83 / 46, 44 / 45; weighted 256^2 grid 230 / 700, 125 / 372, 68 / 204:
+//     by the estimates above;
+//   general products, 512 sources, a batch of 32 / 64 / 128 / 256 / 512 columns
+//     against a source: directed R-MAT 16, weights <= 255, 15 / 17 / 20 / 31 / 56 against
+//     3.3, R-MAT 18 58 / 67 / 98 / 153 / 293 against 9.8; uniform n = 100 000, k = 8,
+//     64 / 160 / 320 columns 9.1 / 22 / 43 against 4.5;
+//   small graphs, R-MAT 12 (a source 0.22 ms), 152 sources on 10 / 20 / 40 blocks
+//     3.3 / 1.3, 1.6 / 1.2, 0.8 / 2.4, 512 sources on 5 / 24 / 47 22.7 / 2.9, 4.6 /
+//     2.9, 2.4 / 2.5; 48 sources on 11 0.9 / 1.2;
+//   levels, uniform n = 60 000, k = 8, 152 sources on 76 blocks 1.9 / 3.9.
+static bool cut_by_source(const DevGraph& g, int path, int32_t nsrc, int blocks, int nb) {
+  const int64_t waves = ((int64_t)nsrc + blocks - 1) / blocks, batches = ((int64_t)nsrc + nb - 1) / nb;
+  if (path == MFBC_PATH_DIST) return dist_source_us(g, nsrc, blocks) < dist_steps_us(g, nsrc, nb);
+  if (path == MFBC_PATH_GENERAL) return waves <= ((has_hubs(g) ? 4 : 0) + nb / 32) * batches;
+  if (path == MFBC_PATH_SMALL) return blocks >= 64 || waves <= 6;
+  return waves <= 3;
+}
+
 static int tuned_slot(int path) {
   return path == MFBC_PATH_LEVEL ? 0 : path == MFBC_PATH_GENERAL ? 1 : path == MFBC_PATH_DIST ? 2 : 3;
 }
@@ -434,26 +458,59 @@ static mfbc_status make_plan(const mfbc_graph* G, int32_t nsrc, int mode, const 
   const bool small = path == MFBC_PATH_SMALL && !(opt && (opt->flags & MFBC_OPT_TEST_STALL));
   const bool open_level = path == MFBC_PATH_LEVEL && !G->tuned_path && !G->tuned_nb[0] &&
                           (!opt || (opt->path == MFBC_PATH_AUTO && !(opt->flags & MFBC_OPT_TEST_SMALL_ROUNDS)));
-  const bool can_source = !hooked && g.nnz < (1ll << 31) && (path == MFBC_PATH_DIST || small || (open_general && general_by_source(g, INT32_MAX)) ||
-                                                  (open_level && level_by_source(g, 1)));
+  const bool can_source = !hooked && g.nnz < (1ll << 31) &&
+                          (path == MFBC_PATH_DIST || small || (open_general && general_by_source(g, INT32_MAX)) ||
+                           (open_level && level_by_source(g, 1)));
   const bool by_source = can_source && (small || (path == MFBC_PATH_DIST    ? dist_by_source(g, nsrc)
                                                   : path == MFBC_PATH_LEVEL ? level_by_source(g, nsrc)
                                                                             : general_by_source(g, nsrc)));
-  // A source plan is cut down to fewer blocks where its scratch does not fit; the
-  // family's kernels take over when not even one block's does.
-  auto fit_source = [&](int nb, size_t room) {
-    if (p->total <= room) return;
-    const size_t rest = p->total - p->src.slot_bytes * (size_t)p->src.slots;
-    const int most = room > rest ? (int)((room - rest) / p->src.slot_bytes) : 0;
-    plan_bytes(g, path, nb, nsrc, mode, host_io, p, true, std::max(most, 1));
-    if (p->total > room) plan_bytes(g, path, nb, nsrc, mode, host_io, p);
+  // The family's kernels at the widest batch up to `top` that fits the room, or
+  // at exactly `top`.
+  auto family = [&](int top, int gran, size_t room, bool fixed) {
+    Plan q;
+    // (the persistent small-graph kernel runs batches side by side: 128 columns per
+    // batch leave it several batches to spread over its block groups)
+    if (path == MFBC_PATH_SMALL && !fixed && !G->tuned_nb[tuned_slot(path)]) top = std::min(top, 128);
+    for (int b = top;; b -= gran) {
+      plan_bytes(g, path, b, nsrc, mode, host_io, &q);
+      if (fixed || q.total <= room || b == gran) return q;
+    }
   };
-  // The family's kernels do not fit a caller's workspace: the source kernel may
-  // (a workspace sized for more sources, where the rule chose it).
-  auto try_source = [&](int nb, size_t room) {
-    if (!can_source || p->by_source || p->total <= room) return;
-    plan_bytes(g, path, nb, nsrc, mode, host_io, p, true);
-    fit_source(nb, room);
+  // The source kernel with at most `top` columns, its blocks cut down to what fits
+  // the room (one at least; staging rows take half of it at most).
+  auto source = [&](int top, int gran, size_t room, bool fixed) {
+    Plan q;
+    for (int b = top;; b -= gran) {
+      plan_bytes(g, path, b, nsrc, mode, host_io, &q, true);
+      if (fixed || q.total <= room || 2 * q.extra_bytes <= room || b == gran) break;
+    }
+    while (q.total > room && q.src.slots > 1) {            // (fewer blocks keep fewer copies of lambda, too)
+      const size_t copies = sizeof(double) * (size_t)q.copies * g.n;
+      const size_t rest = q.total - q.src.slot_bytes * (size_t)q.src.slots - copies;
+      const size_t fit = room > rest ? (room - rest) / q.src.slot_bytes : 1;
+      const size_t with = room > rest + copies ? (room - rest - copies) / q.src.slot_bytes : 1;
+      // as many as fit without copies, then as many as fit with those they keep
+      const size_t most = std::max<size_t>(1, std::min<size_t>(fit < (size_t)q.src.slots ? fit : with, (size_t)q.src.slots - 1));
+      plan_bytes(g, path, q.nb, nsrc, mode, host_io, &q, true, (int)most);
+    }
+    return q;
+  };
+  // One of the two within the room.
+  auto choose = [&](int top, int gran, size_t room, bool fixed) {
+    const bool given = opt && opt->workspace;
+    if (!by_source) {
+      *p = family(top, gran, room, fixed);
+      // (a workspace sized for more sources, where the rule chose the source kernel)
+      if (!can_source || !given || p->total <= room) return;
+      const Plan q = source(top, gran, room, fixed);
+      if (q.total <= room) *p = q;
+      return;
+    }
+    *p = source(top, gran, room, fixed);
+    const int blocks = mode == 1 && host_io ? std::min(p->src.slots, p->nb) : p->src.slots;
+    if (p->total <= room && blocks >= std::min(nsrc, 152)) return;
+    const Plan q = family(top, gran, room, fixed);
+    if (p->total > room || (q.total <= room && !cut_by_source(g, path, nsrc, blocks, q.nb))) *p = q;
   };
   // the level kernels move 128 columns (four 32-column words) at a time
   const int gran = path == MFBC_PATH_LEVEL ? 128 : 32;
@@ -465,20 +522,25 @@ static mfbc_status make_plan(const mfbc_graph* G, int32_t nsrc, int mode, const 
   if (path == MFBC_PATH_LEVEL && (int64_t)g.n * (maxnb / 128) >= (1ll << 31))
     return fail(MFBC_ERR_INVALID, "graph too large for the level kernels' 31-bit pair row indices");
   if (req > 0) {
-    int nb = (req + gran - 1) / gran * gran;
+    const int nb = (req + gran - 1) / gran * gran;
     if (nb > maxnb) return fail(MFBC_ERR_INVALID, "n_b too large for this path (max " + std::to_string(maxnb) + ")");
-    plan_bytes(g, path, nb, nsrc, mode, host_io, p, by_source);
-    // the narrowest width, which callers short of memory come down to, asks for
-    // no more state than 24 bytes per vertex and column
-    if (by_source && nb == gran) fit_source(nb, p->extra_bytes + 24ull * (size_t)g.n * nb + (size_t)(64 << 10));
-    if (opt->workspace) {
-      if (by_source) fit_source(nb, opt->workspace_bytes);
-      else try_source(nb, opt->workspace_bytes);
-    } else if (by_source && p->total > G->ws_bytes) {      // the cached scratch would grow: within the device's room
+    size_t room = SIZE_MAX;
+    if (opt->workspace) room = opt->workspace_bytes;
+    else if (by_source) {                                  // the cached scratch would grow: within the device's room
+      plan_bytes(g, path, nb, nsrc, mode, host_io, p, true);
       size_t fr = 0, tot = 0;
-      if (cudaMemGetInfo(&fr, &tot) == cudaSuccess) fit_source(nb, (size_t)(0.80 * (double)(fr + G->ws_bytes)));
+      if (p->total <= G->ws_bytes) room = G->ws_bytes;
+      else if (cudaMemGetInfo(&fr, &tot) == cudaSuccess) room = (size_t)(0.80 * (double)(fr + G->ws_bytes));
       else cudaGetLastError();
     }
+    // the narrowest width, which callers short of memory come down to, asks for
+    // no more than the family's kernels do there (or 24 bytes per vertex and column)
+    if (by_source && nb == gran) {
+      const Plan f = family(nb, gran, room, true);
+      plan_bytes(g, path, nb, nsrc, mode, host_io, p, true);
+      room = std::min(room, std::max(f.total, p->extra_bytes + (size_t)24 * (size_t)g.n * nb + (size_t)(64 << 10)));
+    }
+    choose(nb, gran, room, true);
     return MFBC_OK;
   }
   // auto: widest batch (<= number of sources, <= the tuned width) whose
@@ -491,25 +553,8 @@ static mfbc_status make_plan(const mfbc_graph* G, int32_t nsrc, int mode, const 
     if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) { cudaGetLastError(); return fail(MFBC_ERR_CUDA, "cudaMemGetInfo failed"); }
     budget = (size_t)(0.80 * (double)(fr + G->ws_bytes));
   }
-  // the persistent small-graph kernel runs batches side by side: 128 columns
-  // per batch leave it several batches to spread over its block groups
-  const int widest = tuned > 0 ? tuned : (path == MFBC_PATH_SMALL && !by_source ? 128 : maxnb);
-  int nb = std::min(widest, std::max(gran, (nsrc + gran - 1) / gran * gran));
-  if (by_source) {
-    int b = nb;
-    for (;; b -= gran) {
-      plan_bytes(g, path, b, nsrc, mode, host_io, p, true);
-      if (p->total <= budget || b == gran) break;
-    }
-    fit_source(b, budget);
-    if (p->by_source) return MFBC_OK;
-  }
-  while (true) {
-    plan_bytes(g, path, nb, nsrc, mode, host_io, p);
-    if (p->total <= budget || nb == gran) break;
-    nb -= gran;
-  }
-  if (opt && opt->workspace) try_source(nb, budget);
+  const int widest = tuned > 0 ? tuned : maxnb;
+  choose(std::min(widest, std::max(gran, (nsrc + gran - 1) / gran * gran)), gran, budget, false);
   return MFBC_OK;
 }
 

@@ -71,3 +71,59 @@ def test_few_sources_of_weighted_graphs(name):
         assert np.array_equal(d, wd) and np.array_equal(s, ws)
     finally:
         G.close()
+
+
+# graph, sources, n_b, path, by source?  (n_b = 32 leaves the source kernel a few
+# blocks, 64 a block a column)
+def _unit_rmat():
+    return gg.rmat(12, 8, seed=7)
+
+
+NARROW_ROUTES = {
+    "dist_uniform_32": (lambda: gg.erdos_renyi(50000, 16, weights=(1, 20), seed=8), 48, 32, mfbc.PATH_AUTO, False),
+    "dist_uniform_64": (lambda: gg.erdos_renyi(50000, 16, weights=(1, 20), seed=8), 64, 64, mfbc.PATH_AUTO, True),
+    "dist_lattice_32": (lambda: gg.grid2d(200, weights=(1, 16), seed=9), 48, 32, mfbc.PATH_AUTO, True),
+    "general_uniform_32": (lambda: gg.erdos_renyi(50000, 8, weights=(1, 255), seed=10), 300, 32, mfbc.PATH_AUTO, False),
+    "general_hubs_64": (lambda: gg.rmat(15, 16, directed=True, weights=(1, 255), seed=10), 300, 64, mfbc.PATH_AUTO, True),
+    "small_32_many": (_unit_rmat, 1000, 32, mfbc.PATH_SMALL, False),
+    "small_32_few": (_unit_rmat, 8, 32, mfbc.PATH_SMALL, True),
+    "small_64": (_unit_rmat, 1000, 64, mfbc.PATH_SMALL, True),
+}
+
+
+def by_source(prof):
+    if prof["path"] == mfbc.PATH_SMALL:          # (the persistent kernel counts one step a batch)
+        return prof["fwd_iters"] != prof["batches"]
+    return not any(k in prof["kernels"] for k in ("dist_mfbr", "mfbf_accumulate", "level_mfbf_gather"))
+
+
+@pytest.mark.parametrize("name", NARROW_ROUTES)
+def test_narrow_batches_and_short_workspaces(name):
+    import torch
+    make, k, n_b, path, want_source = NARROW_ROUTES[name]
+    g = make()
+    srcs = gg.sample_sources(g, k, seed=11)
+    want = oracle.bc(g, srcs)
+    wd, ws, _ = oracle.sssp(g, srcs[:40])
+    G = mfbc.Graph.from_csr(g)
+    try:
+        lam, prof = G.bc(srcs, n_b=n_b, path=path, profile=True)
+        assert by_source(prof) == want_source
+        close(lam, want)
+        # the same calls in a workspace of the size asked for, and n_b = 0 in it
+        work = torch.empty(G.workspace_size(k, 0, n_b=n_b, path=path), dtype=torch.uint8, device="cuda")
+        lam, prof = G.bc(srcs, n_b=n_b, path=path, workspace=work, profile=True)
+        assert by_source(prof) == want_source
+        close(lam, want)
+        close(G.bc(srcs, path=path, workspace=work), want)
+        for rows in (1, 40):
+            work = torch.empty(G.workspace_size(rows, 1, n_b=n_b, path=path), dtype=torch.uint8, device="cuda")
+            d, s = G.sssp(srcs[:rows], n_b=n_b, path=path, workspace=work)
+            assert np.array_equal(d, wd[:rows]) and np.array_equal(s, ws[:rows])
+        cut = k // 3
+        lists = [torch.from_numpy(x).cuda() for x in (srcs[:cut], srcs[cut:])]
+        cols = sum((len(x) + 31) // 32 * 32 for x in lists)
+        work = torch.empty(G.workspace_size(cols, 2, n_b=n_b, path=path), dtype=torch.uint8, device="cuda")
+        close(G.bc_multi(lists, n_b=n_b, path=path, workspace=work).cpu().numpy().sum(0), want)
+    finally:
+        G.close()
