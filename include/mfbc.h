@@ -75,7 +75,11 @@ typedef enum {
                                   else the level kernels; distance kernels for weights
                                   <= 128 when no in- or out-degree exceeds max(64, 4x the
                                   average degree); general kernels otherwise (or the family
-                                  mfbc_autotune chose) */
+                                  mfbc_autotune chose).  Calls of the level family with few
+                                  sources on small graphs, and of the general family with
+                                  weights <= 1024 and no accumulator named, run one block per
+                                  source where that is faster; the profile's path stays the
+                                  family's */
 #define MFBC_PATH_GENERAL 1    /* force the general (any integer weight) kernels */
 #define MFBC_PATH_LEVEL   2    /* require the unit-weight level kernels (INVALID if weighted) */
 #define MFBC_PATH_DIST    3    /* distance-ordered kernels for small integer weights, one block
@@ -280,7 +284,9 @@ typedef struct {
  * widths that do not fit the device are skipped.  With opt->path == AUTO a
  * weighted graph tries both the general and (weights <= 4096) the distance
  * kernels and later AUTO calls use the faster family; another path restricts
- * the search to it.  Each candidate runs twice (the first call untimed).
+ * the search to it.  Later AUTO calls on the level family may still run one
+ * block per source (see MFBC_PATH_AUTO), with fewer sources than nsrc where the
+ * search timed both.  Each candidate runs twice (the first call untimed).
  * Later calls on this handle with opt->n_b == 0 use at most the tuned width
  * (no cap when the fastest width was the widest one tried), and the general
  * kernels use the tuned arcs per step (without tuning: 8 when the average

@@ -26,6 +26,7 @@ struct mfbc_graph {
   int tuned_nb[4] = {0, 0, 0, 0};   // level, general, distance, small-graph family
   int tuned_arcs = 0;
   int tuned_path = 0;               // kernel family for MFBC_PATH_AUTO (0 = by weights)
+  int level_from = INT32_MAX;       // sources from which the level kernels beat the source kernel
   int force_arcs = 0;
   int tuned_accum = 0;              // general kernels' accumulator for MFBC_ACCUM_AUTO (0 = per product)
 };
@@ -453,10 +454,13 @@ static mfbc_status make_plan(const mfbc_graph* G, int32_t nsrc, int mode, const 
   }
   // may the source kernel take the call, and does the rule choose it?
   const bool hooked = opt && (opt->flags & MFBC_OPT_TEST_FAMILY_KERNELS);
+  // (tuning a family chooses among its own kernels, which is no reason not to run
+  // by source; tuning under AUTO has timed the source kernel against the general
+  // products, and against the level kernels on graphs of the small family's size)
   const bool open_general = path == MFBC_PATH_GENERAL && (!opt || (opt->path == MFBC_PATH_AUTO && !opt->accumulator)) &&
-                            !G->tuned_path && !G->tuned_arcs && !G->tuned_accum && !G->force_arcs;
+                            !G->tuned_path;
   const bool small = path == MFBC_PATH_SMALL && !(opt && (opt->flags & MFBC_OPT_TEST_STALL));
-  const bool open_level = path == MFBC_PATH_LEVEL && !G->tuned_path && !G->tuned_nb[0] &&
+  const bool open_level = path == MFBC_PATH_LEVEL && nsrc < G->level_from &&
                           (!opt || (opt->path == MFBC_PATH_AUTO && !(opt->flags & MFBC_OPT_TEST_SMALL_ROUNDS)));
   const bool can_source = !hooked && g.nnz < (1ll << 31) &&
                           (path == MFBC_PATH_DIST || small || (open_general && general_by_source(g, INT32_MAX)) ||
@@ -1330,6 +1334,12 @@ extern "C" mfbc_status mfbc_autotune(mfbc_graph* G, const int32_t* sources, int3
     const int gran = level ? 128 : 32;
     const int cols = (nsrc + gran - 1) / gran * gran;
     while (widths.size() > 1 && widths.back() > cols) widths.pop_back();
+    // The source kernel takes the small family's calls whatever their width (but
+    // the narrowest, short of memory): the widest goes first, and a narrower one
+    // has to be 5 % faster, or the timer's noise would choose a width that later
+    // calls stage their rows in.
+    const int widest = widths.back();
+    if (path == MFBC_PATH_SMALL) std::reverse(widths.begin(), widths.end());
     // general kernels: atomic products walking 1 or 8 arcs per step, the
     // segmented products, the hash-combined products, and the per-product
     // choice between atomic and segmented
@@ -1360,9 +1370,9 @@ extern "C" mfbc_status mfbc_autotune(mfbc_graph* G, const int32_t* sources, int3
           return s;
         }
         tried++;
-        if (best_nb == 0 || ms < best) {
+        if (best_nb == 0 || ms < (path == MFBC_PATH_SMALL && best_path == path ? 0.95 : 1.0) * best) {
           best = ms; best_nb = nb; best_arcs = a; best_path = path; best_accum = var.accum;
-          best_widest = nb == widths.back();
+          best_widest = nb == widest;
         }
       }
   }
@@ -1375,7 +1385,10 @@ extern "C" mfbc_status mfbc_autotune(mfbc_graph* G, const int32_t* sources, int3
     G->tuned_arcs = best_arcs;
     G->tuned_accum = best_accum;
   }
-  if (req_path == MFBC_PATH_AUTO) G->tuned_path = best_path;
+  if (req_path == MFBC_PATH_AUTO) {
+    G->tuned_path = best_path;
+    G->level_from = paths.size() > 1 && best_path == MFBC_PATH_LEVEL ? nsrc : INT32_MAX;
+  }
   out->n_b = best_nb;
   out->path = best_path;
   out->arcs = best_arcs;
