@@ -462,7 +462,7 @@ static mfbc_status make_plan(const mfbc_graph* G, int32_t nsrc, int mode, const 
   const bool small = path == MFBC_PATH_SMALL && !(opt && (opt->flags & MFBC_OPT_TEST_STALL));
   const bool open_level = path == MFBC_PATH_LEVEL && nsrc < G->level_from &&
                           (!opt || (opt->path == MFBC_PATH_AUTO && !(opt->flags & MFBC_OPT_TEST_SMALL_ROUNDS)));
-  const bool can_source = !hooked && g.nnz < (1ll << 31) &&
+  const bool can_source = !hooked && source_graph(g) && (g.unit || g.pk) &&
                           (path == MFBC_PATH_DIST || small || (open_general && general_by_source(g, INT32_MAX)) ||
                            (open_level && level_by_source(g, 1)));
   const bool by_source = can_source && (small || (path == MFBC_PATH_DIST    ? dist_by_source(g, nsrc)

@@ -218,23 +218,30 @@ __global__ void k_pack_arcs(const int32_t* __restrict__ col, const int32_t* __re
 // Column and weight of a weighted graph's arc in one word, for the source
 // kernel (half the bytes and one load an arc).  They always fit: distances are
 // int32, so n * w_max < 2^31, and with n > 2^(cb-1), w_max >= 2^(wb-1) the bits
-// cb + wb are at most 32.
-static mfbc_status pack_arcs(DevGraph* g, cudaStream_t st, std::string* err) {
-  int cb = 1, wb = 1;
+// cb + wb are at most 32.  Graphs that no call runs by source (see source_graph)
+// go without them, and so do graphs that the device has no room left for them:
+// their calls run on the families' kernels.
+static void pack_arcs(DevGraph* g, cudaStream_t st) {
+  int cb = 1;
   while ((1ll << cb) < g->n) cb++;
-  while ((1ll << wb) <= g->wmax) wb++;
-  if (!g->w) return MFBC_OK;
-  if (cb + wb > 32) { *err = "column and weight of an arc do not fit in 32 bits"; return MFBC_ERR_OVERFLOW; }
+  bool room = g->w && source_graph(*g);
+  if (room && !g->pk) room = dev_alloc(g, &g->pk, (size_t)g->nnz, nullptr) == MFBC_OK;
+  if (room && g->directed && !g->pk_t) {
+    room = dev_alloc(g, &g->pk_t, (size_t)g->nnz, nullptr) == MFBC_OK;
+    if (!room && g->nnz > JOINED_ARCS) {         // (the last allocation made: pk)
+      cudaFree(g->pk);
+      g->owned.pop_back();
+    }
+  }
+  if (!room) {
+    g->pk = g->pk_t = nullptr;
+    return;
+  }
   g->pk_bits = cb;
   const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>((g->nnz + 255) / 256, 152 * 16));
-  if (!g->pk) TRY(dev_alloc(g, &g->pk, (size_t)g->nnz, err));
   k_pack_arcs<<<blocks, 256, 0, st>>>(g->col, g->w, g->nnz, cb, g->pk);
   if (!g->directed) g->pk_t = g->pk;
-  else {
-    if (!g->pk_t) TRY(dev_alloc(g, &g->pk_t, (size_t)g->nnz, err));
-    k_pack_arcs<<<blocks, 256, 0, st>>>(g->col_t, g->w_t, g->nnz, cb, g->pk_t);
-  }
-  return MFBC_OK;
+  else k_pack_arcs<<<blocks, 256, 0, st>>>(g->col_t, g->w_t, g->nnz, cb, g->pk_t);
 }
 
 // About how many arcs the far ends of the graph are apart, from the breadth-first
@@ -638,7 +645,7 @@ mfbc_status graph_build(int32_t n, int64_t nnz, const int64_t* h_rowptr, const i
     g->col_t = g->col;
     g->w_t = g->w;
   }
-  TRY(pack_arcs(g, st, err));
+  pack_arcs(g, st);
   // (calls on the graph may come on any stream: everything is there at return)
   MFBC_CUDA_TRY(cudaStreamSynchronize(st), err);
   MFBC_CUDA_TRY(cudaGetLastError(), err);

@@ -51,7 +51,7 @@ struct DevGraph {
   int64_t* rowptr_t = nullptr;     // CSR of A^T (in-arcs); aliases CSR when undirected
   int32_t* col_t = nullptr;
   int32_t* w_t = nullptr;
-  uint32_t* pk = nullptr;          // A's arcs as column | weight << pk_bits (nullptr when unit)
+  uint32_t* pk = nullptr;          // A's arcs as column | weight << pk_bits (nullptr: unit, or not packed)
   uint32_t* pk_t = nullptr;        //   and those of A^T (aliases pk when undirected)
   int pk_bits = 0;
   double hops = 0.0;               // weighted: estimated arcs across the graph (0: not estimated)
@@ -223,6 +223,11 @@ void dist_carve(Carver& c, int32_t n, int nb, int B, DistState& s);
 
 // Source path: one block per source, for weighted graphs in order of distance
 // value and for small unit-weight graphs by levels.  See source.cu.
+// Sizes that its kernels are written for: weights within the buckets, 32-bit arc
+// counts and queue positions (and, weighted, an n that its families take).
+inline bool source_graph(const DevGraph& g) {
+  return g.nnz < (1ll << 31) && (g.unit || (g.wmax + 1 <= DIST_MAX_BUCKETS && (uint64_t)g.n * 128u <= 0xffffffffull));
+}
 struct SourcePlan {
   bool unit = false;     // by levels, 64-bit counts
   int dm = 0, am = 0;    // where tau lives, how arcs are stored (DM_*, AM_* of source.cu)
