@@ -96,6 +96,10 @@ typedef struct mfbc_graph mfbc_graph;   /* opaque, device resident */
  * the algorithmic (compulsory) DRAM traffic of those launches under the
  * model documented beside each kernel. */
 #define MFBC_MAX_KSTATS 24
+/* One kernel of a call.  The one-block-per-source kernel, whose single launch is
+ * MFBF and MFBr of every source, appears as "small_persistent" on MFBC_PATH_SMALL,
+ * as "dist_mfbf" on MFBC_PATH_DIST (the family's step kernels always have a
+ * "dist_mfbr" beside it) and as "source_bc" on the level and general families. */
 typedef struct {
   char name[40];
   uint64_t launches;
@@ -115,7 +119,7 @@ typedef struct {
                                   settled pairs, distance 0 excepted; one block per source:
                                   as fwd_iters, MFBr running inside the same kernel) */
   int32_t n_b;                 /* batch width used */
-  int32_t path;                /* MFBC_PATH_GENERAL, MFBC_PATH_LEVEL or MFBC_PATH_DIST */
+  int32_t path;                /* the family: MFBC_PATH_GENERAL, _LEVEL, _DIST or _SMALL */
   uint64_t stat[4];            /* with MFBC_OPT_COUNT_BYTES, level kernels: (neighbour, word)
                                   pairs gathered by MFBF / MFBr, values gathered by MFBF / MFBr */
 } mfbc_profile;
@@ -262,7 +266,7 @@ mfbc_status mfbc_bc_multi_device(const mfbc_graph* g, const int32_t* sources, in
 /* Result of mfbc_autotune. */
 typedef struct {
   int32_t n_b;            /* fastest batch width found */
-  int32_t path;           /* MFBC_PATH_LEVEL, MFBC_PATH_GENERAL or MFBC_PATH_DIST */
+  int32_t path;           /* MFBC_PATH_LEVEL, _GENERAL, _DIST or _SMALL */
   int32_t arcs;           /* general kernels: arcs walked per step (1 or 8); 0 on the level kernels */
   int32_t tried;          /* configurations timed */
   double ms_per_source;   /* wall time of the fastest configuration per source */

@@ -889,7 +889,9 @@ mfbc_status source_path(Run& R, RunCtx& rc, const int32_t* d_src, int32_t nsrc, 
                         int32_t* stage_d, double* stage_s, uint32_t* warn, int64_t* fi, int64_t* bi) {
   const DevGraph& g = *rc.g;
   const Plan& P = R.plan;
-  const KId id = P.src.unit ? K_SMALL : K_DP_FWD;
+  // (booked under the main kernel's label of the families that this kernel serves,
+  // see mfbc_kernel_stat; under its own for the two that have kernels of their own)
+  const KId id = P.path == MFBC_PATH_SMALL ? K_SMALL : P.path == MFBC_PATH_DIST ? K_DP_FWD : K_SOURCE;
   SourceState ss, sw;
   Carver c1(R.ws, R.ws_bytes), c2(R.ws, R.ws_bytes);
   const size_t copied = (size_t)P.copies * g.n;

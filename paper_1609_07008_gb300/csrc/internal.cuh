@@ -72,7 +72,7 @@ enum KId {
   K_FILL = 0, K_SEED, K_RELAX_MIN, K_RELAX_TIE, K_ACCUM, K_COUNTERS, K_PROPAGATE, K_FINAL,
   K_LAMBDA, K_CLEAR, K_LVL_FWD, K_LVL_VISIT, K_LVL_BWD, K_LVL_HUB, K_LVL_RESET, K_OUTPUT,
   K_LVL_FWD_G, K_LVL_BWD_G, K_LVL_SPLIT, K_DP_FWD, K_DP_BWD, K_SMALL, K_PULL_FWD, K_PULL_BWD,
-  K_HASH_MIN, K_HASH_TIE, K_HASH_PROP, K_NUM
+  K_HASH_MIN, K_HASH_TIE, K_HASH_PROP, K_SOURCE, K_NUM
 };
 
 // Bits of Counters::flags, set by kernels and read by the host drivers.
