@@ -395,10 +395,20 @@ static bool general_by_source(const DevGraph& g, int32_t nsrc) {
 // two are close up to 152 sources (n = 100 000, k = 8 1.4 / 1.5, 2.2 / 1.7, 2.9 /
 // 2.4) or the level kernels win (n = 20 000, k = 60 0.7 / 1.2, 1.1 / 1.3, 1.4 /
 // 1.3; R-MAT 15 0.9 / 0.9, 1.2 / 1.3, 1.6 / 1.4), unless the graph is sparse
-// enough to be deep (n = 600 000, k = 2 5.8 / 4.5, 14 / 5.4, 21 / 10).
+// enough to be deep (n = 620 000, k = 2, 1 / 8 / 152 sources 4.9 / 4.7, 9.0 / 4.9, 20 /
+// 11; n = 400 000, k = 3 2.9 / 4.0, 4.8 / 4.0, 12 / 10, directed 3.1 / 4.9, 4.9 / 5.0,
+// 11 / 12).  Dense graphs have three or
+// four levels (n = 9000, k = 66, 1 / 152 sources 0.54 / 0.83, 0.82 / 0.83; k = 33
+// 0.57 / 0.40, 0.82 / 0.43), and the source kernel walks a directed graph's rows
+// both ways (n = 32 768, k = 18, 1 / 32 / 152 sources 0.84 / 1.01, 1.07 / 1.08, 1.32 /
+// 1.11).
 static bool level_by_source(const DevGraph& g, int32_t nsrc) {
-  return g.nnz <= (g.nnz <= 3 * (int64_t)g.n ? 1250000 : 600000) &&
-         (nsrc <= 152 || (int64_t)nsrc * g.nnz <= 130000000);
+  const int64_t n = g.n;
+  int64_t most = 600000;
+  if (g.nnz <= 2 * n || (g.nnz <= 3 * n && nsrc >= 8 && !(g.directed && nsrc > 64))) most = 1250000;
+  else if (g.nnz >= 48 * n) most = 420000;
+  else if (g.directed && nsrc < 32 && g.nnz > 4 * n) most = 400000;
+  return g.nnz <= most && (nsrc <= 152 || (int64_t)nsrc * g.nnz <= 130000000);
 }
 
 // The rules above compare the sides at full width.  With little scratch, or a
@@ -464,7 +474,7 @@ static mfbc_status make_plan(const mfbc_graph* G, int32_t nsrc, int mode, const 
                           (!opt || (opt->path == MFBC_PATH_AUTO && !(opt->flags & MFBC_OPT_TEST_SMALL_ROUNDS)));
   const bool can_source = !hooked && source_graph(g) && (g.unit || g.pk) &&
                           (path == MFBC_PATH_DIST || small || (open_general && general_by_source(g, INT32_MAX)) ||
-                           (open_level && level_by_source(g, 1)));
+                           (open_level && level_by_source(g, 32)));
   const bool by_source = can_source && (small || (path == MFBC_PATH_DIST    ? dist_by_source(g, nsrc)
                                                   : path == MFBC_PATH_LEVEL ? level_by_source(g, nsrc)
                                                                             : general_by_source(g, nsrc)));

@@ -73,6 +73,33 @@ def test_few_sources_of_weighted_graphs(name):
         G.close()
 
 
+# unit weights past the small family: graph, sources, by the level kernels?
+LEVEL_ROUTES = {
+    "dense_one_source": (lambda: gg.erdos_renyi(9000, 65, seed=12), 1, True),
+    "dense_fewer_arcs": (lambda: gg.erdos_renyi(9000, 33, seed=13), 1, False),
+    "directed_one_source": (lambda: gg.erdos_renyi(16384, 35, directed=True, seed=14), 1, True),
+    "sparse_one_source": (lambda: gg.erdos_renyi(400000, 3, seed=15), 1, True),
+    "sparse_more_sources": (lambda: gg.erdos_renyi(400000, 3, seed=15), 40, False),
+    "deep_one_source": (lambda: gg.grid2d(256, seed=16), 1, False),
+}
+
+
+@pytest.mark.parametrize("name", LEVEL_ROUTES)
+def test_few_sources_of_unit_weight_graphs(name):
+    make, k, levels = LEVEL_ROUTES[name]
+    g = make()
+    g = gg.CSRGraph(n=g.n, rowptr=g.rowptr, col=g.col, w=None, directed=g.directed)
+    srcs = gg.sample_sources(g, k, seed=17)
+    G = mfbc.Graph.from_csr(g)
+    try:
+        lam, prof = G.bc(srcs, profile=True)
+        assert prof["path"] == mfbc.PATH_LEVEL
+        assert ("level_mfbf_gather" in prof["kernels"]) == levels
+        close(lam, oracle.bc(g, srcs))
+    finally:
+        G.close()
+
+
 # graph, sources, n_b, path, by source?  (n_b = 32 leaves the source kernel a few
 # blocks, 64 a block a column)
 def _unit_rmat():
