@@ -83,11 +83,12 @@ typedef enum {
 #define MFBC_PATH_GENERAL 1    /* force the general (any integer weight) kernels */
 #define MFBC_PATH_LEVEL   2    /* require the unit-weight level kernels (INVALID if weighted) */
 #define MFBC_PATH_DIST    3    /* distance-ordered kernels for small integer weights, one block
-                                  per source or, for few sources of a large graph, the whole
-                                  device per distance step (INVALID when the largest weight exceeds 4096); n_b is at
+                                  per source or, for few sources of a large graph or little
+                                  scratch, the whole device per distance step (INVALID when the largest weight exceeds 4096); n_b is at
                                   most 4096 and n * n_b stays below 2^32 */
 #define MFBC_PATH_SMALL   4    /* small unit-weight graphs: every source of the call in one
-                                  launch, one block per source (INVALID if weighted) */
+                                  launch, one block per source or, with little scratch, batches
+                                  on groups of blocks (INVALID if weighted) */
 
 typedef struct mfbc_graph mfbc_graph;   /* opaque, device resident */
 

@@ -27,8 +27,9 @@
 //
 // These kernels spread one step of all sources over the whole device.  The
 // source kernel (source.cu: a block per source, no launch per step) takes
-// every call but few sources of a large graph; the rule and both sides'
-// figures are in api.cu.
+// every call but few sources of a large graph and narrow batches or short
+// scratch that leave it too few blocks; the rules (dist_by_source, cut_by_source)
+// and both sides' figures are in api.cu.
 #include <algorithm>
 
 #include "internal.cuh"

@@ -313,9 +313,10 @@ struct RowLanes {
 // A warp reads one row eight times before it needs the first, or, with up to
 // NARROW_W words (256 columns), several rows at once, four times.  MFBF / MFBr
 // pair kernels of a call, one row against several: R-MAT 18, 100 sources 0.77 /
-// 0.61 -> 0.67 / 0.50 ms, 256 sources 0.85 / 0.70 -> 0.77 / 0.61, 384 (two rows) 0.96 /
-// 0.79 -> 0.95 / 0.80; R-MAT 20, 128 sources 3.00 / 2.48 -> 2.49 / 1.91.  (A kernel of
-// its own: as a branch, the wide form lost 5-20 %.)
+// 0.61 -> 0.67 / 0.50 ms, 256 sources 0.85 / 0.70 -> 0.77 / 0.61; R-MAT 20, 128 sources
+// 3.00 / 2.48 -> 2.49 / 1.91.  (A kernel of its own: as a branch, the wide form lost
+// 5-20 %.  Tried and not kept: two rows at once up to 512 columns, 384 sources 0.96 /
+// 0.79 -> 0.95 / 0.80.)
 constexpr int NARROW_W = 8;
 template <bool NARROW>
 __device__ __forceinline__ uint32_t stage_rows(WarpSmem& sm, int nm, int W, const RowLanes& rl,
@@ -1555,7 +1556,7 @@ mfbc_status level_batch(RunCtx& rc, LevelState& s, const int32_t* d_src_batch, i
       k_lvl_cursor<<<1, 1, 0, st>>>(s.ctr, 0);
     }
     if (flags & (FLAG_LEVEL_LIST | FLAG_COUNT_WRAP)) {
-      // list capacity exceeded (bit 0) or a path count passed 2^64 (bit 3):
+      // list capacity exceeded (bit 0) or a path count reached 2^58 (bit 3):
       // the general kernels redo this batch; rows of vertices missing from
       // the overflowed list may hold bits, so every mask is cleared
       k_clear_flag_bits<<<1, 1, 0, st>>>(&s.ctr->flags, FLAG_LEVEL_LIST | FLAG_COUNT_WRAP);

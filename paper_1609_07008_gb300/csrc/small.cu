@@ -36,9 +36,12 @@
 // depth limit); its MFBr is skipped, so it adds nothing to lambda here.
 //
 // The source kernel (source.cu) runs these graphs 2.4 to 10 times faster (a
-// block per source: no barrier across blocks) and takes every call it can; this
-// kernel keeps graphs of 2^31 arcs and more, and calls with the hook that makes
-// a device wait run out (MFBC_OPT_TEST_STALL): it is the one with such waits.
+// block per source: no barrier across blocks) and takes every call that leaves it
+// enough blocks.  This kernel keeps calls of many sources at n_b = 32 or in a short
+// workspace (cut_by_source in api.cu: R-MAT 12, 512 sources in 11 MB 2.9 ms against
+// 4.6 on 24 blocks), graphs of 2^31 arcs and more, and the calls of two test hooks:
+// MFBC_OPT_TEST_FAMILY_KERNELS, and MFBC_OPT_TEST_STALL, which makes a device wait
+// run out (it is the kernel with such waits).
 #include <algorithm>
 
 #include "dfloat.cuh"

@@ -911,7 +911,10 @@ void source_plan(const DevGraph& g, int cols, bool unit, bool wide, SourcePlan& 
     p.o_dag = c.off; c.take<uint32_t>((size_t)p.dcap * (n <= 65536 ? 1 : 2));
     return c.off;
   };
-  // unit-weight graphs: at most 256 MB of block states, but two sources an SM
+  // unit-weight graphs: two sources an SM, or as many as 256 MB of block states
+  // hold.  (Two take what they need: 152 sources of a graph of 10^7 vertices and
+  // 10^6 arcs 49 GB, where the level kernels' state takes 38 GB and the call 3.7 ms
+  // instead of 1.3.  Calls cut the blocks down to the scratch there is.)
   if (p.unit)
     per_sm = std::min(per_sm, std::max<int64_t>(2, (256ll << 20) / (int64_t)layout(false) / SRC_SMS));
   const int64_t ring = (int64_t)src_al16((size_t)p.B * 4) + (int64_t)src_al16((size_t)p.B * p.scap * 4);
@@ -939,7 +942,7 @@ void source_plan(const DevGraph& g, int cols, bool unit, bool wide, SourcePlan& 
       p.dm = form[f];
       db = bytes;
       p.threads = room(1024, bytes) >= 1 ? 1024 : 512;
-      while (p.threads > 128 && 2 * room(p.threads / 2, bytes) > 2 * room(p.threads, bytes) &&
+      while (p.threads > 128 && room(p.threads / 2, bytes) > room(p.threads, bytes) &&
              room(p.threads / 2, bytes) <= share)
         p.threads /= 2;
     }
