@@ -320,6 +320,19 @@ static int default_path(const DevGraph& g) {
   return MFBC_PATH_GENERAL;
 }
 
+// The columns of a call: its sources and, where several requests are packed, what
+// rounds each of them up to a 32-column word.  The source kernel runs the sources
+// alone.  The general products take a word of one source for as long as a full
+// one (uniform n = 100 000, k = 8, weights <= 255, 1 / 4 / 8 / 16 requests of one
+// source 3.3 / 8.9 / 19 / 38 ms; 16 sources of one request 5.2).  The distance kernels
+// take about twice as long for a source that shares no word (uniform n = 10^6,
+// k = 8, weights <= 20, 8 / 16 requests of one 16 / 30, 8 / 24 sources of one 11 / 21).
+struct Columns {
+  int32_t sources, all;
+  bool several() const { return all > (sources + 31) / 32 * 32; }
+  int32_t steps() const { return several() ? (int32_t)std::min<int64_t>(2 * (int64_t)sources, all) : sources; }
+};
+
 // The source kernel (source.cu) or the kernels of the family, for the distance
 // kernels and for calls of the general kernels that leave the choice open
 // (MFBC_PATH_AUTO, untuned, no accumulator named).
@@ -367,10 +380,11 @@ static double dist_source_us(const DevGraph& g, int32_t nsrc, int blocks) {
                      arc * (double)g.nnz;
   return one * ((nsrc + blocks - 1) / blocks);
 }
-static bool dist_by_source(const DevGraph& g, int32_t nsrc) {
-  if (g.n < (1 << 15) || nsrc > 40) return true;
+// (steps: the sources as the distance kernels feel them, see Columns)
+static bool dist_by_source(const DevGraph& g, int32_t nsrc, int32_t steps) {
+  if (g.n < (1 << 15) || steps > 40) return true;
   const int32_t k = std::max(nsrc, 1);
-  return dist_source_us(g, k, k) < dist_steps_us(g, k, 64);
+  return dist_source_us(g, k, k) < dist_steps_us(g, std::max(steps, 1), 64);
 }
 // The general kernels' time goes with their 15-25 Bellman-Ford products (0.1-0.3
 // ms each and up) whatever the weights are, the source kernel's with the
@@ -427,9 +441,9 @@ static bool level_by_source(const DevGraph& g, int32_t nsrc) {
 //     3.3 / 1.3, 1.6 / 1.2, 0.8 / 2.4, 512 sources on 5 / 24 / 47 22.7 / 2.9, 4.6 /
 //     2.9, 2.4 / 2.5; 48 sources on 11 0.9 / 1.2;
 //   levels, uniform n = 60 000, k = 8, 152 sources on 76 blocks 1.9 / 3.9.
-static bool cut_by_source(const DevGraph& g, int path, int32_t nsrc, int blocks, int nb) {
-  const int64_t waves = ((int64_t)nsrc + blocks - 1) / blocks, batches = ((int64_t)nsrc + nb - 1) / nb;
-  if (path == MFBC_PATH_DIST) return dist_source_us(g, nsrc, blocks) < dist_steps_us(g, nsrc, nb);
+static bool cut_by_source(const DevGraph& g, int path, const Columns& c, int blocks, int nb) {
+  const int64_t waves = ((int64_t)c.sources + blocks - 1) / blocks, batches = ((int64_t)c.all + nb - 1) / nb;
+  if (path == MFBC_PATH_DIST) return dist_source_us(g, c.sources, blocks) < dist_steps_us(g, c.steps(), nb);
   if (path == MFBC_PATH_GENERAL) return waves <= ((has_hubs(g) ? 4 : 0) + nb / 32) * batches;
   if (path == MFBC_PATH_SMALL) return blocks >= 64 || waves <= 6;
   return waves <= 3;
@@ -439,7 +453,9 @@ static int tuned_slot(int path) {
   return path == MFBC_PATH_LEVEL ? 0 : path == MFBC_PATH_GENERAL ? 1 : path == MFBC_PATH_DIST ? 2 : 3;
 }
 
-static mfbc_status make_plan(const mfbc_graph* G, int32_t nsrc, int mode, const mfbc_options* opt,
+// nsrc: the columns to plan for (mode 2: each request rounded up to 32); asked: the
+// sources among them.
+static mfbc_status make_plan(const mfbc_graph* G, int32_t nsrc, int32_t asked, int mode, const mfbc_options* opt,
                              bool host_io, Plan* p) {
   const DevGraph& g = G->g;
   int path = opt ? opt->path : MFBC_PATH_AUTO;
@@ -470,14 +486,16 @@ static mfbc_status make_plan(const mfbc_graph* G, int32_t nsrc, int mode, const 
   const bool open_general = path == MFBC_PATH_GENERAL && (!opt || (opt->path == MFBC_PATH_AUTO && !opt->accumulator)) &&
                             !G->tuned_path;
   const bool small = path == MFBC_PATH_SMALL && !(opt && (opt->flags & MFBC_OPT_TEST_STALL));
-  const bool open_level = path == MFBC_PATH_LEVEL && nsrc < G->level_from &&
+  const bool open_level = path == MFBC_PATH_LEVEL && asked < G->level_from &&
                           (!opt || (opt->path == MFBC_PATH_AUTO && !(opt->flags & MFBC_OPT_TEST_SMALL_ROUNDS)));
   const bool can_source = !hooked && source_graph(g) && (g.unit || g.pk) &&
                           (path == MFBC_PATH_DIST || small || (open_general && general_by_source(g, INT32_MAX)) ||
                            (open_level && level_by_source(g, 32)));
-  const bool by_source = can_source && (small || (path == MFBC_PATH_DIST    ? dist_by_source(g, nsrc)
-                                                  : path == MFBC_PATH_LEVEL ? level_by_source(g, nsrc)
-                                                                            : general_by_source(g, nsrc)));
+  const Columns cols{asked, nsrc};
+  const bool by_source = can_source &&
+                         (small || (path == MFBC_PATH_DIST    ? dist_by_source(g, asked, cols.steps())
+                                    : path == MFBC_PATH_LEVEL ? level_by_source(g, asked)
+                                                              : general_by_source(g, cols.several() ? nsrc : asked)));
   // The family's kernels at the widest batch up to `top` that fits the room, or
   // at exactly `top`.
   auto family = [&](int top, int gran, size_t room, bool fixed) {
@@ -495,7 +513,7 @@ static mfbc_status make_plan(const mfbc_graph* G, int32_t nsrc, int mode, const 
   auto source = [&](int top, int gran, size_t room, bool fixed) {
     Plan q;
     for (int b = top;; b -= gran) {
-      plan_bytes(g, path, b, nsrc, mode, host_io, &q, true);
+      plan_bytes(g, path, b, asked, mode, host_io, &q, true);
       if (fixed || q.total <= room || 2 * q.extra_bytes <= room || b == gran) break;
     }
     while (q.total > room && q.src.slots > 1) {            // (fewer blocks keep fewer copies of lambda, too)
@@ -505,7 +523,7 @@ static mfbc_status make_plan(const mfbc_graph* G, int32_t nsrc, int mode, const 
       const size_t with = room > rest + copies ? (room - rest - copies) / q.src.slot_bytes : 1;
       // as many as fit without copies, then as many as fit with those they keep
       const size_t most = std::max<size_t>(1, std::min<size_t>(fit < (size_t)q.src.slots ? fit : with, (size_t)q.src.slots - 1));
-      plan_bytes(g, path, q.nb, nsrc, mode, host_io, &q, true, (int)most);
+      plan_bytes(g, path, q.nb, asked, mode, host_io, &q, true, (int)most);
     }
     return q;
   };
@@ -522,9 +540,9 @@ static mfbc_status make_plan(const mfbc_graph* G, int32_t nsrc, int mode, const 
     }
     *p = source(top, gran, room, fixed);
     const int blocks = mode == 1 && host_io ? std::min(p->src.slots, p->nb) : p->src.slots;
-    if (p->total <= room && blocks >= std::min(nsrc, 152)) return;
+    if (p->total <= room && blocks >= std::min(asked, 152)) return;
     const Plan q = family(top, gran, room, fixed);
-    if (p->total > room || (q.total <= room && !cut_by_source(g, path, nsrc, blocks, q.nb))) *p = q;
+    if (p->total > room || (q.total <= room && !cut_by_source(g, path, cols, blocks, q.nb))) *p = q;
   };
   // the level kernels move 128 columns (four 32-column words) at a time
   const int gran = path == MFBC_PATH_LEVEL ? 128 : 32;
@@ -541,7 +559,7 @@ static mfbc_status make_plan(const mfbc_graph* G, int32_t nsrc, int mode, const 
     size_t room = SIZE_MAX;
     if (opt->workspace) room = opt->workspace_bytes;
     else if (by_source) {                                  // the cached scratch would grow: within the device's room
-      plan_bytes(g, path, nb, nsrc, mode, host_io, p, true);
+      plan_bytes(g, path, nb, asked, mode, host_io, p, true);
       size_t fr = 0, tot = 0;
       if (p->total <= G->ws_bytes) room = G->ws_bytes;
       else if (cudaMemGetInfo(&fr, &tot) == cudaSuccess) room = (size_t)(0.80 * (double)(fr + G->ws_bytes));
@@ -551,7 +569,7 @@ static mfbc_status make_plan(const mfbc_graph* G, int32_t nsrc, int mode, const 
     // no more than the family's kernels do there (or 24 bytes per vertex and column)
     if (by_source && nb == gran) {
       const Plan f = family(nb, gran, room, true);
-      plan_bytes(g, path, nb, nsrc, mode, host_io, p, true);
+      plan_bytes(g, path, nb, asked, mode, host_io, p, true);
       room = std::min(room, std::max(f.total, p->extra_bytes + (size_t)24 * (size_t)g.n * nb + (size_t)(64 << 10)));
     }
     choose(nb, gran, room, true);
@@ -579,7 +597,7 @@ extern "C" mfbc_status mfbc_workspace_size(const mfbc_graph* G, int32_t nsrc, in
   Plan p;
   mfbc_options o = opt ? *opt : mfbc_options{};
   o.workspace = nullptr;
-  mfbc_status s = make_plan(G, nsrc, mode, &o, mode != 2, &p);
+  mfbc_status s = make_plan(G, nsrc, nsrc, mode, &o, mode != 2, &p);
   if (s) return s;
   *bytes = p.total;
   return MFBC_OK;
@@ -1234,7 +1252,7 @@ mfbc_status entry(const mfbc_graph* Gc, const int32_t* sources, int32_t nsrc, in
     for (int32_t r = 0; r < nreq; r++) cols += (req_off[r + 1] - req_off[r] + 31) / 32 * 32;
     plan_cols = (int32_t)std::min<int64_t>(cols, 0x7fffffff);
   }
-  mfbc_status s = make_plan(G, plan_cols, mode, opt, host_io, &R.plan);
+  mfbc_status s = make_plan(G, plan_cols, nsrc, mode, opt, host_io, &R.plan);
   if (s) return s;
   s = get_workspace(R);
   if (s) return s;

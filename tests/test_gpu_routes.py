@@ -154,3 +154,25 @@ def test_narrow_batches_and_short_workspaces(name):
         close(G.bc_multi(lists, n_b=n_b, path=path, workspace=work).cpu().numpy().sum(0), want)
     finally:
         G.close()
+
+
+def test_requests_of_few_sources_count_as_few():
+    # four requests of one source are 128 packed columns, eight 256
+    import torch
+    for make, r, kernel, steps in ((lambda: gg.erdos_renyi(1 << 17, 64, weights=(1, 4), seed=18), 4, "dist_mfbr", True),
+                                   (lambda: gg.erdos_renyi(60000, 9, seed=19), 8, "level_mfbf_gather", False)):
+        g = make()
+        srcs = gg.sample_sources(g, r, seed=20)
+        G = mfbc.Graph.from_csr(g)
+        try:
+            lists = [torch.from_numpy(srcs[i:i + 1]).cuda() for i in range(r)]
+            lam, prof = G.bc_multi(lists, profile=True)
+            assert (kernel in prof["kernels"]) == steps
+            # in the workspace that the columns ask for, whichever kernels that is for
+            for n_b in (0, 32, 256):
+                work = torch.empty(G.workspace_size(32 * r, 2, n_b=n_b), dtype=torch.uint8, device="cuda")
+                close(G.bc_multi(lists, n_b=n_b, workspace=work).cpu().numpy(), lam.cpu().numpy())
+            for i in range(r):
+                close(lam[i].cpu().numpy(), oracle.bc(g, srcs[i:i + 1]))
+        finally:
+            G.close()
