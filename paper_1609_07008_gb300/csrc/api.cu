@@ -1364,12 +1364,12 @@ extern "C" mfbc_status mfbc_autotune(mfbc_graph* G, const int32_t* sources, int3
     const int gran = level ? 128 : 32;
     const int cols = (nsrc + gran - 1) / gran * gran;
     while (widths.size() > 1 && widths.back() > cols) widths.pop_back();
-    // The source kernel takes the small family's calls whatever their width (but
-    // the narrowest, short of memory): the widest goes first, and a narrower one
-    // has to be 5 % faster, or the timer's noise would choose a width that later
-    // calls stage their rows in.
+    // The source kernel takes the small family's calls whatever their width: the
+    // widest goes first and stands for all that it takes, or the timer's noise would
+    // choose a width that later calls stage their rows in.
     const int widest = widths.back();
     if (path == MFBC_PATH_SMALL) std::reverse(widths.begin(), widths.end());
+    bool by_source = false;
     // general kernels: atomic products walking 1 or 8 arcs per step, the
     // segmented products, the hash-combined products, and the per-product
     // choice between atomic and segmented
@@ -1400,7 +1400,17 @@ extern "C" mfbc_status mfbc_autotune(mfbc_graph* G, const int32_t* sources, int3
           return s;
         }
         tried++;
-        if (best_nb == 0 || ms < (path == MFBC_PATH_SMALL && best_path == path ? 0.95 : 1.0) * best) {
+        if (path == MFBC_PATH_SMALL) {
+          std::lock_guard<std::mutex> lock(G->mu);
+          Plan plan;
+          const bool again = by_source;
+          by_source = make_plan(G, nsrc, nsrc, 0, &o, true, &plan) == MFBC_OK && plan.by_source;
+          if (by_source && again) {
+            if (best_path == path) best = std::min(best, ms);
+            continue;
+          }
+        }
+        if (best_nb == 0 || ms < best) {
           best = ms; best_nb = nb; best_arcs = a; best_path = path; best_accum = var.accum;
           best_widest = nb == widest;
         }
