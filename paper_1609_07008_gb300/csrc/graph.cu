@@ -250,11 +250,13 @@ static void pack_arcs(DevGraph* g, cudaStream_t st) {
 // radius, as on lattices and road networks, and is carried on with that power;
 // otherwise it grows by a factor a level.  Only api.cu's choice between kernels of
 // equal results depends on it, and only for graphs of HOPS_ROWS vertices and more.
-// It takes 40-80 us on the host.  (A ball of 4096 would tell three-dimensional
-// lattices from graphs of degree 2 that double, but takes 150-300 us.)
+// It takes 10-20 us on the host, of the 400 and more of creating such a graph.  (A
+// ball of 4096 would tell three-dimensional lattices from graphs of degree 2 that
+// double, but takes ten times as long; one of 256 takes lattices of degree 8 for
+// random graphs.)
 constexpr int32_t HOPS_ROWS = 1 << 15;
 static double estimate_hops(int32_t n, const int64_t* rp, const int32_t* col, const std::vector<int32_t>& roots) {
-  constexpr int BALL = 1024, SLOTS = 4 * BALL, ARCS = 1 << 14;
+  constexpr int BALL = 512, SLOTS = 4 * BALL, ARCS = 1 << 13;
   const size_t target = BALL;
   std::vector<int32_t> slots, order;
   std::vector<size_t> size, best;      // vertices within l levels
@@ -263,7 +265,8 @@ static double estimate_hops(int32_t n, const int64_t* rp, const int32_t* col, co
     order.clear();
     size.clear();
     auto visit = [&](int32_t v) {
-      uint32_t h = ((uint32_t)v * 2654435769u) >> 20;                     // 12 bits
+      if (v < 0 || v >= n) return;
+      uint32_t h = ((uint32_t)v * 2654435769u) >> 21;                     // 11 bits
       while (slots[h] != v && slots[h] != -1) h = (h + 1) % SLOTS;
       if (slots[h] == v) return;
       slots[h] = v;
@@ -591,6 +594,9 @@ mfbc_status graph_build(int32_t n, int64_t nnz, const int64_t* h_rowptr, const i
     g->items_in = g->items_out;
     g->hot_in = g->hot_out;
   }
+  // (on the host while the device works; the arcs are not known to be valid yet.
+  // Rows of hundreds of arcs settle the choice without it.)
+  if (h_w && n >= HOPS_ROWS && g->max_deg <= std::max<int64_t>(64, 4 * (nnz / n))) g->hops = estimate_hops(n, h_rowptr, h_col, g->landmarks);
   MFBC_CUDA_TRY(cudaMemcpyAsync(&f, d_f, sizeof(f), cudaMemcpyDeviceToHost, st), err);
   MFBC_CUDA_TRY(cudaStreamSynchronize(st), err);
   MFBC_CUDA_TRY(cudaGetLastError(), err);
@@ -605,8 +611,7 @@ mfbc_status graph_build(int32_t n, int64_t nnz, const int64_t* h_rowptr, const i
     return MFBC_ERR_OVERFLOW;
   }
   g->unit = !f.non_unit;
-  if (!g->unit && n >= HOPS_ROWS && g->wmax + 1 <= DIST_MAX_BUCKETS)
-    g->hops = estimate_hops(n, h_rowptr, h_col, g->landmarks);
+  if (g->unit) g->hops = 0.0;
   if (g->unit && g->w) { g->w = nullptr; g->pk = nullptr; }   // all ones: treat as unweighted (arrays still owned)
   if (g->directed) {
     // A^T by a stable counting sort on the host: rows of A^T are sorted by
